@@ -190,7 +190,7 @@ __device__ __forceinline__ void vt_item(const R* XFz, int v, const RefConst<P, R
       R s = R(0);
 #pragma unroll
       for (int a = 0; a < RP::NFN; ++a) s += ps[a] * Xs[a];
-      if (valid) trF[(static_cast<size_t>(m * Dm::NQT + f0 + q) * 8 + v) * Z + z] = s * iJF[f0 + q];
+      if (valid) trF[(static_cast<size_t>(m * Dm::NQT + f0 + q) * Z + z) * 8 + v] = s * iJF[f0 + q];
     }
   } else {
     constexpr int le = e - 6;
@@ -203,7 +203,7 @@ __device__ __forceinline__ void vt_item(const R* XFz, int v, const RefConst<P, R
       R s = R(0);
 #pragma unroll
       for (int a = 0; a < RP::NEN; ++a) s += ps[a] * Xs[a];
-      if (valid) trE[(static_cast<size_t>(m * 12 * Dm::NS + idx) * 8 + v) * Z + z] = s * iJE[idx];
+      if (valid) trE[(static_cast<size_t>(m * 12 * Dm::NS + idx) * Z + z) * 8 + v] = s * iJE[idx];
     }
   }
 }

@@ -3,7 +3,9 @@
 
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -569,6 +571,31 @@ int geo_stage_flops(geo_mesh_t m, double* fl, int64_t* units) {
   return GEO_OK;
 }
 
+// The traces are stored [point][Z][8]; the debug calls hand them over as
+// [point][8][Z].  Reorders n host values in place, to the caller's order or to the
+// stored one; false when the scratch row cannot be allocated.
+static bool swap_trace_order(double* host, int64_t n, int64_t Z, bool to_caller) {
+  std::unique_ptr<double[]> row(new (std::nothrow) double[8 * Z]);
+  if (!row) return false;
+  for (double* h = host; h < host + n; h += 8 * Z) {
+    for (int64_t z = 0; z < Z; ++z)
+      for (int v = 0; v < 8; ++v) {
+        if (to_caller) row[v * Z + z] = h[z * 8 + v];
+        else row[z * 8 + v] = h[v * Z + z];
+      }
+    std::memcpy(h, row.get(), 8 * Z * sizeof(double));
+  }
+  return true;
+}
+// a copy of the caller's n trace values in the stored order (null: no memory)
+static std::unique_ptr<double[]> stored_traces(const double* host, int64_t n, int64_t Z) {
+  std::unique_ptr<double[]> c(new (std::nothrow) double[n]);
+  if (!c) return nullptr;
+  std::memcpy(c.get(), host, n * sizeof(double));
+  if (!swap_trace_order(c.get(), n, Z, false)) return nullptr;
+  return c;
+}
+
 int geo_debug_buffer(geo_mesh_t m, int which, double* host, int64_t count) {
   if (!m || !host) return fail(GEO_ERR_ARG, "bad arguments");
   const geo::Dims& d = m->T.d;
@@ -598,6 +625,8 @@ int geo_debug_buffer(geo_mesh_t m, int which, double* host, int64_t count) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "debug copy");
+  if ((which == 2 || which == 3) && !swap_trace_order(host, n, Z, true))
+    return fail(GEO_ERR_OOM, "host allocation failed");
   return GEO_OK;
 }
 
@@ -712,6 +741,12 @@ int geo_debug_set_buffer(geo_mesh_t m, int which, const double* host, int64_t co
   int rc = debug_buffer_slot(m, which, &dst, &n);
   if (rc != GEO_OK) return rc;
   if (count != n) return fail(GEO_ERR_ARG, "geo_debug_set_buffer: count must equal the buffer size");
+  std::unique_ptr<double[]> stored;
+  if (which == 2 || which == 3) {
+    stored = stored_traces(host, n, m->T.Z);
+    if (!stored) return fail(GEO_ERR_OOM, "host allocation failed");
+    host = stored.get();
+  }
   cudaError_t e = cudaMemcpyAsync(dst, host, n * sizeof(double), cudaMemcpyHostToDevice, m->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->st);
   if (e != cudaSuccess) return cuda_fail(e, "debug copy");
@@ -755,6 +790,12 @@ int geo_debug_stage_vjp(geo_mesh_t m, int stage, double dt, const double* U, con
     default: return fail(GEO_ERR_ARG, "geo_debug_stage_vjp: stage must be WENO, ADER, FACE or EDGE");
   }
   if (n_out != want_out || n_in != want_in) return fail(GEO_ERR_ARG, "geo_debug_stage_vjp: wrong buffer sizes");
+  std::unique_ptr<double[]> stored;
+  if (stage == geo::ST_ADER) {
+    stored = stored_traces(g_out, n_out, Z);
+    if (!stored) return fail(GEO_ERR_OOM, "host allocation failed");
+    g_out = stored.get();
+  }
   // the zone cotangents: a zero incoming one, and the WENO stage's output
   double* gU0 = nullptr;
   double* gU = nullptr;
@@ -796,6 +837,8 @@ int geo_debug_stage_vjp(geo_mesh_t m, int stage, double dt, const double* U, con
   cudaFree(gU0);
   cudaFree(gU);
   if (e != cudaSuccess) return cuda_fail(e, "geo_debug_stage_vjp");
+  if ((stage == geo::ST_FACE || stage == geo::ST_EDGE) && !swap_trace_order(g_in, n_in, Z, true))
+    return fail(GEO_ERR_OOM, "host allocation failed");
   return GEO_OK;
 }
 

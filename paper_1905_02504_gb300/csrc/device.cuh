@@ -86,8 +86,8 @@ struct DevState {
   double* phi;   // [F]
   void* Wc;      // (R) [8*NC1][Z] WENO-AO Taylor coefficients
   void* Bp;      // (R) [NQmax][F]  nodal normal B per face (canonical orientation)
-  void* trF;     // (R) [(M-1)*NQT*8][Z] predictor states at the zone's face points
-  void* trE;     // (R) [(M-1)*12*NS*8][Z] predictor states at the zone's edge points
+  void* trF;     // (R) [(M-1)*NQT][Z][8] predictor states at the zone's face points
+  void* trE;     // (R) [(M-1)*12*NS][Z][8] predictor states at the zone's edge points
   double* Ff;    // [8][F] time-integrated face fluxes (FP64 accumulation)
   double* Ee;    // [E]   time-integrated edge EMFs (FP64 accumulation)
   double* red;   // reduction scratch

@@ -437,9 +437,9 @@ __global__ void __launch_bounds__(TPB) k_ader(const DevTables T, double* __restr
           for (int v = 0; v < 8; ++v) acc[v] += w * Uh[m][i][v];
         }
         const R iJ = R(1) / JF[idx];
-        R* out = trF + (static_cast<size_t>((m - 1) * NQT + idx) * 8) * Z + z;
 #pragma unroll
-        for (int v = 0; v < 8; ++v) out[v * Z] = acc[v] * iJ;
+        for (int v = 0; v < 8; ++v) acc[v] *= iJ;
+        st8(trF + trF_at<P>(z, m, idx, Z), acc);
       }
     }
   const R* JE = BT.JE + static_cast<size_t>(c) * 12 * NS;
@@ -461,9 +461,9 @@ __global__ void __launch_bounds__(TPB) k_ader(const DevTables T, double* __restr
           for (int v = 0; v < 8; ++v) acc[v] += w * Uh[m][i][v];
         }
         const R iJ = R(1) / JE[idx];
-        R* out = trE + (static_cast<size_t>((m - 1) * 12 * NS + idx) * 8) * Z + z;
 #pragma unroll
-        for (int v = 0; v < 8; ++v) out[v * Z] = acc[v] * iJ;
+        for (int v = 0; v < 8; ++v) acc[v] *= iJ;
+        st8(trE + trE_at<P>(z, m, idx, Z), acc);
       }
 }
 
@@ -491,16 +491,18 @@ __global__ void __launch_bounds__(TPB) k_pos_traces(const DevTables T, const dou
     if (pass == 2 && !(th < R(1))) break;
 #pragma unroll 1
     for (int t = 0; t < NPF + NPE; ++t) {
-      R* base = (t < NPF) ? trF + (static_cast<size_t>(t) * 8) * Z + z
-                          : trE + (static_cast<size_t>(t - NPF) * 8) * Z + z;
+      // point t over all Gauss times (trF_at / trE_at)
+      R* base = (t < NPF) ? trF + (static_cast<size_t>(t) * Z + z) * 8
+                          : trE + (static_cast<size_t>(t - NPF) * Z + z) * 8;
       R s[8];
-#pragma unroll
-      for (int v = 0; v < 8; ++v) s[v] = base[v * Z];
+      ld8(base, s);
       if (pass == 0) pos_rho(s, Uz, eps_r, th_r);
       else if (pass == 1) pos_p(s, Uz, th_r, gR, pbar, eps_p, th_p);
-      else
+      else {
 #pragma unroll
-        for (int v = 0; v < 8; ++v) base[v * Z] = Uz[v] + th * (s[v] - Uz[v]);
+        for (int v = 0; v < 8; ++v) s[v] = Uz[v] + th * (s[v] - Uz[v]);
+        st8(base, s);
+      }
     }
   }
 }
@@ -948,7 +950,7 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
           const R ij = valid2 ? R(1) / JF[idx] : R(1);
 #pragma unroll
           for (int v = 0; v < 8; ++v) s[v] *= ij;
-          out = trF + (static_cast<size_t>(t) * 8) * Z + z2;
+          out = trF + (static_cast<size_t>(t) * Z + z2) * 8;
         } else {
           const int tt = t - NPF, m = tt / (12 * NS), idx = tt % (12 * NS), le = idx / NS;
 #pragma unroll
@@ -966,7 +968,7 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
           const R ij = valid2 ? R(1) / JE[idx] : R(1);
 #pragma unroll
           for (int v = 0; v < 8; ++v) s[v] *= ij;
-          out = trE + (static_cast<size_t>(tt) * 8) * Z + z2;
+          out = trE + (static_cast<size_t>(tt) * Z + z2) * 8;
         }
         if (!valid2) continue;
         if constexpr (POS) {
@@ -986,8 +988,7 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
             for (int v = 0; v < 8; ++v) s[v] = Uz[v] + th * (s[v] - Uz[v]);
           }
         }
-#pragma unroll
-        for (int v = 0; v < 8; ++v) out[v * Z] = s[v];
+        st8(out, s);
       }
       if constexpr (POS) __syncthreads();
     }
@@ -1028,17 +1029,11 @@ __global__ void __launch_bounds__(TPB) k_face_flux(const DevTables T, const R* _
       R nx = gs * nv[0], ny = gs * nv[1], nz = gs * nv[2];
       const R W = static_cast<R>(wt * T.WF[static_cast<size_t>(fi.cg) * NQT + ig] * s2);
       R uL[8], uR[8];
-      if (fi.zL >= 0) {
-        const R* src = trF + trF_at<P>(fi.zL, m, foff<P>(fi.lfL) + q, Z);
-#pragma unroll
-        for (int v = 0; v < 8; ++v) uL[v] = src[v * Z];
-      }
+      if (fi.zL >= 0) ld8(trF + trF_at<P>(fi.zL, m, foff<P>(fi.lfL) + q, Z), uL);
       if (fi.zR >= 0) {
         int ql = q;
         if (fi.se >= 0) ql = T.se_perm[fi.se * Dm::NQS + q];
-        const R* src = trF + trF_at<P>(fi.zR, m, foff<P>(fi.lfR) + ql, Z);
-#pragma unroll
-        for (int v = 0; v < 8; ++v) uR[v] = src[v * Z];
+        ld8(trF + trF_at<P>(fi.zR, m, foff<P>(fi.lfR) + ql, Z), uR);
       }
       if (fi.zL < 0) {
 #pragma unroll
@@ -1139,9 +1134,7 @@ __global__ void __launch_bounds__(TPB) k_edge_emf(const DevTables T, const R* __
         R u[8] = {R(1), R(0), R(0), R(0), R(1), R(0), R(0), R(0)};
         if (j < nz) {
           const int sl = revs[j] ? NS - 1 - s : s;
-          const R* src = trE + trE_at<P>(zs[j], m, les[j] * NS + sl, Z);
-#pragma unroll
-          for (int v = 0; v < 8; ++v) u[v] = src[v * Z];
+          ld8(trE + trE_at<P>(zs[j], m, les[j] * NS + sl, Z), u);
         }
         const Prim<R> w = to_prim(u, g);
         ir[j] = R(1) / u[0];
