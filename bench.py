@@ -100,20 +100,20 @@ def workload_name(a):
 
 
 def default_schedule(order, fp32=False):
-    """The library's default predictor schedule: the variable-layout team at
-    orders 2 and 3 and for the FP32-bulk form, the node team for FP64 at order 4."""
-    return 2 if (order <= 3 or fp32) else 1
+    """The library's default predictor schedule: the variable team."""
+    return 2
 
 
 def kernel_name(stage, pred, positivity=False, order=4, fp32=False):
     """Name of the kernel that runs a stage (the predictor stage has three
-    schedules; the variable-layout one runs the node team when positivity is on)."""
+    schedules; the variable team with positivity on has its own kernel at order 4
+    and at order 3 in FP64, and runs the node team's elsewhere)."""
     name = "k_" + stage
     if stage == "ader":
         if pred is None:
             pred = default_schedule(order, fp32)
-        if pred == 2 and not positivity:
-            name += "_vt"
+        if pred == 2 and (not positivity or order == 4 or (order == 3 and not fp32)):
+            name += "_ring"
         elif pred != 0:
             name += "_team"
     return name
@@ -297,14 +297,13 @@ def reference_arm(a):
     print(json.dumps(line), flush=True)
 
 
-PREDICTOR_SOURCES = ("device.cuh", "mhd_device.cuh", "ader_vt.cuh")
+PREDICTOR_SOURCES = ("device.cuh", "mhd_device.cuh", "ader_ring.cuh")
 
 
 def predictor_fingerprint():
     """sha256 prefix of the predictor kernels' source: the node-team section of
-    kernels.cu (from the team sizes to the face-flux stage), ader_vt.cuh, the
-    device headers they use and the generator of the compiled pattern
-    (refpattern.py, whose row groups set the variable team's work split).
+    kernels.cu (from the team sizes to the face-flux stage), ader_ring.cuh, the
+    device headers they use and the generator of the compiled pattern.
     Edits elsewhere in the library leave it unchanged."""
     import hashlib
     csrc = os.path.join(ROOT, "paper_1905_02504_gb300", "csrc")

@@ -176,10 +176,7 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   D.E_rad = T.E_rad;
   D.gamma = 5.0 / 3.0;
   D.positivity = 0;
-  // default schedule: the variable-layout team where it measured faster (orders
-  // 2, 3, and the FP32-bulk form at order 4), the node team for FP64 at order 4
-  // (3 % faster there)
-  D.predictor = (order <= 3 || prec == GEO_FP32_BULK) ? GEO_PRED_VAR_TEAM : GEO_PRED_NODE_TEAM;
+  D.predictor = GEO_PRED_VAR_TEAM;  // the fastest schedule at every order and form
   D.riemann = GEO_RIEMANN_HLL;
   std::vector<double> qpow(T.nr + 2);
   for (int k = 0; k < T.nr + 2; ++k) qpow[k] = std::pow(T.q, k);
@@ -211,17 +208,23 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   D.nF = m->upload(T.nF, err);
   D.wF = m->upload(T.wF, err);
   D.WF = m->upload(T.WF, err);
-  // GB and TN transposed per column (team threads read consecutive rows)
+  // per column: the KKT rows of the nodal values and TN transposed (node threads read
+  // consecutive entries, whole 128-byte lines), and the three rows of the zone mean
   const int NR = 3 + 3 * d.N;
-  std::vector<double> GBt(T.GB.size()), TNt(T.TN.size());
+  const size_t ncb = static_cast<size_t>(T.ncol) * d.NBIN;
+  std::vector<double> GBt(ncb * 3 * d.N), GMt(ncb * 3), TNt(T.TN.size());
   for (int c = 0; c < T.ncol; ++c) {
     const size_t g0 = static_cast<size_t>(c) * NR * d.NBIN, t0 = static_cast<size_t>(c) * d.N * d.NC1;
-    for (int r = 0; r < NR; ++r)
-      for (int b = 0; b < d.NBIN; ++b) GBt[g0 + static_cast<size_t>(b) * NR + r] = T.GB[g0 + static_cast<size_t>(r) * d.NBIN + b];
+    const size_t cb = static_cast<size_t>(c) * d.NBIN;
+    for (int b = 0; b < d.NBIN; ++b) {
+      for (int r = 0; r < 3; ++r) GMt[3 * cb + static_cast<size_t>(r) * d.NBIN + b] = T.GB[g0 + static_cast<size_t>(r) * d.NBIN + b];
+      for (int r = 3; r < NR; ++r) GBt[(cb + b) * (NR - 3) + r - 3] = T.GB[g0 + static_cast<size_t>(r) * d.NBIN + b];
+    }
     for (int i = 0; i < d.N; ++i)
       for (int mm = 0; mm < d.NC1; ++mm) TNt[t0 + static_cast<size_t>(mm) * d.N + i] = T.TN[t0 + static_cast<size_t>(i) * d.NC1 + mm];
   }
   D.GB = m->upload(GBt, err);
+  D.GM = m->upload(GMt, err);
   D.TN = m->upload(TNt, err);
   D.J0 = m->upload(T.J0, err);
   D.iJ0 = m->upload(T.iJ0, err);
@@ -262,7 +265,7 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   for (size_t t = 0; t < iJF.size(); ++t) iJF[t] = 1.0 / T.JF[t];
   for (size_t t = 0; t < iJE.size(); ++t) iJE[t] = 1.0 / T.JE[t];
   D.b64 = geo::BulkTables<double>{D.pinvH, D.oct_inv, D.Q,        D.TF,       D.nF,       D.wF,
-                                  D.GB,    D.TN,      D.J0,       D.iJ0,      D.Sm,       D.gcl,
+                                  D.GB,    D.GM,      D.TN,      D.J0,       D.iJ0,      D.Sm,       D.gcl,
                                   D.JF,    D.JE,      D.se_t,     D.se_nang,  D.se_nradL, D.se_nradR,
                                   D.sv_fn, D.sv_t,    m->upload(weta, err), m->upload(iJF, err),
                                   m->upload(iJE, err)};
@@ -279,6 +282,7 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
     b.nF = m->upload_f32(T.nF, err);
     b.wF = m->upload_f32(T.wF, err);
     b.GB = m->upload_f32(GBt, err);
+    b.GM = m->upload_f32(GMt, err);
     b.TN = m->upload_f32(TNt, err);
     b.J0 = m->upload_f32(T.J0, err);
     b.iJ0 = m->upload_f32(T.iJ0, err);

@@ -34,15 +34,22 @@ template <int P, typename R> struct RefConst {
   unsigned char enode[12 * Dim<P>::NEN];
   R R_[Dim<P>::M * Dim<P>::M];
   R Dpat[3 * Dim<P>::NNZ];                      // D^alpha at the compiled pattern (refpattern.h)
+  // ring order of the predictor's contraction and point values (ader_ring.cuh):
+  // place 4 k + q of each node around each axis; point weights of a side face, of
+  // the distinct points of a radial face (corner, middle of a side, centre) and of an
+  // edge on their nodes in ring order; sums over m > 1 of the rows of R
+  unsigned char rpos[3 * Dim<P>::N], tnode[Dim<P>::N];
+  R wS[Dim<P>::NQS * Dim<P>::NFN], wR[3 * Dim<P>::NFN], wEd[Dim<P>::NS * P], Rs[Dim<P>::M - 1];
 };
 
 // Per-column matrices used by the bulk arithmetic, in its type R.  The FP64
 // form points at the FP64 tables; the FP32-bulk form at FP32 copies made once
-// at mesh creation (the FP64 masters stay on the device).  GB and TN are stored
-// transposed on the device, [ncol][NBIN][3+3N] and [ncol][NC1][N], so that the
+// at mesh creation (the FP64 masters stay on the device).  GB (the KKT rows of the
+// nodal values), GM (those of the zone mean) and TN are stored
+// [ncol][NBIN][3N], [ncol][3][NBIN] and [ncol][NC1][N], so that the
 // threads of a node team read consecutive entries.
 template <typename R> struct BulkTables {
-  const R *pinvH, *oct_inv, *Q, *TF, *nF, *wF, *GB, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
+  const R *pinvH, *oct_inv, *Q, *TF, *nF, *wF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
   // edge geometry: unit tangents and face normals at the edge points
   const R *se_t, *se_nang, *se_nradL, *se_nradR, *sv_fn, *sv_t;
   // [ncol] (l_0 / |x_0|)^2 of the column's zones (the same along a self-similar
@@ -69,7 +76,7 @@ struct DevTables {
   const int* st_nb;
   const double* pinvH;
   const int* oct_nb;
-  const double *oct_inv, *Q, *V0, *l0, *S0, *A0, *TF, *nF, *wF, *WF, *GB, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
+  const double *oct_inv, *Q, *V0, *l0, *S0, *A0, *TF, *nF, *wF, *WF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
   const int *col_side_se, *col_side_sgn;
   const int *se_v, *se_col, *se_lf, *se_perm, *se_le, *se_rev;
   const double *se_t, *se_dlw, *se_nang, *se_nradL, *se_nradR;

@@ -18,6 +18,7 @@
 #include "refpattern.h"  // generated at build time (refpattern.py)
 
 #include <cfloat>
+#include <cmath>
 #include <utility>
 #include <vector>
 
@@ -321,14 +322,15 @@ __global__ void __launch_bounds__(TPB) k_ader(const DevTables T, double* __restr
     }
     in[3 * NC + NQT + lf] = static_cast<R>(sg * phi[f] / (T.A0[6 * c + lf] * s2));
   }
-  const R* GB = BT.GB + static_cast<size_t>(c) * (3 + 3 * N) * NBIN;
+  const R* GB = BT.GB + static_cast<size_t>(c) * 3 * N * NBIN;
+  const R* GM = BT.GM + static_cast<size_t>(c) * 3 * NBIN;
   R Uz[8];
 #pragma unroll
   for (int v = 0; v < 5; ++v) Uz[v] = static_cast<R>(U[v * Z + z]);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     R s = R(0);
-    for (int b = 0; b < NBIN; ++b) s += GB[b * (3 + 3 * N) + d] * in[b];
+    for (int b = 0; b < NBIN; ++b) s += GM[d * NBIN + b] * in[b];
     Uz[5 + d] = s;
     U[(5 + d) * Z + z] = static_cast<double>(s);  // Sec. IV.b step 10: zone B <- divergence-free mean
   }
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(TPB) k_ader(const DevTables T, double* __restr
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       R s = R(0);
-      for (int b = 0; b < NBIN; ++b) s += GB[b * (3 + 3 * N) + 3 + d * N + i] * in[b];
+      for (int b = 0; b < NBIN; ++b) s += GB[b * 3 * N + d * N + i] * in[b];
       u[5 + d] = s;
     }
     const R jf = POS ? R(1) : J0[i];
@@ -645,7 +647,7 @@ __device__ __forceinline__ void team_load_inputs(SM& S, const DevTables& T, doub
                                                  const double* __restrict__ phi, const R* __restrict__ Wc,
                                                  const R* __restrict__ Bp, double dt, long long zbase, int tid) {
   using Dm = Dim<P>;
-  constexpr int NC1 = Dm::NC1, NC = Dm::NC, NQT = Dm::NQT, NBIN = Dm::NBIN, NR = 3 + 3 * Dm::N,
+  constexpr int NC1 = Dm::NC1, NC = Dm::NC, NQT = Dm::NQT, NBIN = Dm::NBIN,
                 ZB = Team<P>::ZB, NT = ZB * Dm::N;
   const BulkTables<R>& BT = bulk<R>(T);
   const long long Z = T.Z, F = T.F;
@@ -697,9 +699,9 @@ __device__ __forceinline__ void team_load_inputs(SM& S, const DevTables& T, doub
     const long long z = zbase + zl;
     if (z < Z) {
       const int c = static_cast<int>(z / nr);
-      const R* GB = BT.GB + static_cast<size_t>(c) * NR * NBIN;
+      const R* GM = BT.GM + (static_cast<size_t>(c) * 3 + d) * NBIN;
       R s = R(0);
-      for (int b = 0; b < NBIN; ++b) s += GB[b * NR + d] * S.in[zl][b];
+      for (int b = 0; b < NBIN; ++b) s += GM[b] * S.in[zl][b];
       S.Uz[zl][5 + d] = s;
       if constexpr (WRITE_U) U[(5 + d) * Z + z] = static_cast<double>(s);
       if (d == 0) S.fs[zl] = static_cast<R>(dt / T.qpow[z % nr]);  // one FP64 division per zone
@@ -715,7 +717,7 @@ template <int P, typename R, typename SM>
 __device__ __forceinline__ void team_nodal_values(const SM& S, const BulkTables<R>& BT, int c, int i, int zl,
                                                   bool valid, R* u) {
   using Dm = Dim<P>;
-  constexpr int N = Dm::N, NC1 = Dm::NC1, NBIN = Dm::NBIN, NR = 3 + 3 * Dm::N;
+  constexpr int N = Dm::N, NC1 = Dm::NC1, NBIN = Dm::NBIN;
   if (valid) {
     const R* TN = BT.TN + static_cast<size_t>(c) * N * NC1;
 #pragma unroll
@@ -724,11 +726,11 @@ __device__ __forceinline__ void team_nodal_values(const SM& S, const BulkTables<
       for (int m = 0; m < NC1; ++m) s += TN[m * N + i] * S.W[zl][v * NC1 + m];
       u[v] = s;
     }
-    const R* GB = BT.GB + static_cast<size_t>(c) * NR * NBIN;
+    const R* GB = BT.GB + static_cast<size_t>(c) * 3 * N * NBIN;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       R s = R(0);
-      for (int b = 0; b < NBIN; ++b) s += GB[b * NR + 3 + d * N + i] * S.in[zl][b];
+      for (int b = 0; b < NBIN; ++b) s += GB[b * 3 * N + d * N + i] * S.in[zl][b];
       u[5 + d] = s;
     }
   } else {
@@ -996,6 +998,7 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
 }
 
 #include "ader_vt.cuh"
+#include "ader_ring.cuh"
 
 // ----------------------------------------------------------------------------
 // a4: face fluxes (HLL at face points x Gauss times, FP64 accumulation)
@@ -1435,6 +1438,84 @@ int reduction_blocks(long long n) {
   return static_cast<int>(b);
 }
 
+// Places and weights of the ring order.  The kernels use one set of point weights
+// for all faces and edges, so every face's and edge's own weights are checked
+// against it, node by node; false if the element does not have that symmetry.
+template <int P, typename R>
+bool ring_constants(const Tables& T, RefConst<P, R>& h) {
+  using Dm = Dim<P>;
+  using G = Ring<P>;
+  constexpr int N = Dm::N, NFN = Dm::NFN, PI = G::PI, NU = P == 4 ? 3 : 2, NV = 2;
+  for (int a = 0; a < 3; ++a)
+    for (int q = 0; q < 4; ++q)
+      for (int k = 0; k < G::K; ++k) h.rpos[a * N + G::node(a, q, k)] = static_cast<unsigned char>(4 * k + q);
+  for (int t = 0; t < N; ++t) h.tnode[t] = static_cast<unsigned char>(G::thread_node(t));
+  for (int k = 1; k < Dm::M; ++k) {
+    double s = 0.0;
+    for (int m = 1; m < Dm::M; ++m) s += T.R[k * Dm::M + m];
+    h.Rs[k - 1] = static_cast<R>(s);
+  }
+  double tab[3][Dm::NQS * NFN + 3 * NFN] = {};
+  auto same = [](double a, double b) { return std::fabs(a - b) <= 1e-12; };
+  const int lf_of_q[4] = {2, 1, 3, 0};
+  for (int q = 0; q < 4; ++q) {
+    int nd[NFN];
+    for (int k = 0; k < P; ++k) {
+      nd[k] = G::node(2, q, k);
+      nd[P + k] = G::node(2, (q + 1) & 3, k);
+    }
+    for (int k = 0; k < G::PS; ++k) nd[2 * P + k] = G::node(2, q, P + k);
+    for (int a = 0; a < NU; ++a)
+      for (int b = 0; b < NV; ++b)
+        for (int t = 0; t < NFN; ++t) {
+          const int idx = lf_of_q[q] * Dm::NQS + (q < 2 ? a : NU - 1 - a) * NV + b;
+          const double w = T.psiF[static_cast<size_t>(idx) * N + nd[t]];
+          double& ref = tab[0][(a * NV + b) * NFN + t];
+          if (q == 0) ref = w;
+          else if (!same(ref, w)) return false;
+        }
+    // radial faces
+    const int pa[3] = {G::bit_b(q) * (NU - 1), q == 1 ? 2 : (q == 3 ? 0 : 1), 1};
+    const int pb[3] = {G::bit_c(q) * (NU - 1), q == 0 ? 0 : (q == 2 ? 2 : 1), 1};
+    for (int top = 0; top < 2; ++top) {
+      for (int r = 0; r < 4; ++r) {
+        nd[r] = G::node(2, (q + r) & 3, top * (P - 1));
+        for (int t = 0; t < PI; ++t) nd[4 + r * PI + t] = G::node(2, (q + r) & 3, P + top * PI + t);
+      }
+      for (int w3 = 0; w3 < (P == 4 ? 3 : 1); ++w3)
+        for (int t = 0; t < NFN; ++t) {
+          const int idx = 4 * Dm::NQS + top * Dm::NQR + pa[w3] * NU + pb[w3];
+          const double w = T.psiF[static_cast<size_t>(idx) * N + nd[t]];
+          double& ref = tab[1][w3 * NFN + t];
+          if (q == 0 && top == 0) ref = w;
+          else if (!same(ref, w)) return false;
+        }
+    }
+    // edges: radial edge q, bottom and top edge of face q
+    for (int e = 0; e < 3; ++e) {
+      const int le = e == 0 ? G::edge(2, q) : G::cross_edge(2, q, e - 1);
+      for (int s = 0; s < Dm::NS; ++s)
+        for (int k = 0; k < P; ++k) {
+          int node = G::node(2, q, k);
+          if (e > 0) {
+            const int end = (e - 1) * (P - 1);
+            node = k == 0 ? G::node(2, q, end)
+                          : (k == P - 1 ? G::node(2, (q + 1) & 3, end) : G::node(2, q, P + (e - 1) * PI + k - 1));
+          }
+          const int sp = (e > 0 && q >= 2) ? Dm::NS - 1 - s : s;
+          const double w = T.psiE[(static_cast<size_t>(le) * Dm::NS + sp) * N + node];
+          double& ref = tab[2][s * P + k];
+          if (q == 0 && e == 0) ref = w;
+          else if (!same(ref, w)) return false;
+        }
+    }
+  }
+  for (int t = 0; t < Dm::NQS * NFN; ++t) h.wS[t] = static_cast<R>(tab[0][t]);
+  for (int t = 0; t < 3 * NFN; ++t) h.wR[t] = static_cast<R>(tab[1][t]);
+  for (int t = 0; t < Dm::NS * P; ++t) h.wEd[t] = static_cast<R>(tab[2][t]);
+  return true;
+}
+
 template <int P, typename R>
 cudaError_t upload_reference_constants(const Tables& T) {
   using Dm = Dim<P>;
@@ -1474,6 +1555,7 @@ cudaError_t upload_reference_constants(const Tables& T) {
     for (int t = 0; t < 12 * Dm::NEN; ++t)
       if (T.enode[t] != RP::EN[t]) return cudaErrorInvalidValue;
   }
+  if (!ring_constants(T, h)) return cudaErrorInvalidValue;
   // row form of D^alpha, padded to RL entries per row with zeros (column = the row)
   for (int al = 0; al < 3; ++al) {
     int fill[Dm::N] = {};
@@ -1508,10 +1590,16 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
       k_bperp<P, R><<<grid_for(T.F), TPB, 0, st>>>(T, S.U, S.phi, Wc, Bp);
       break;
     case ST_ADER:
-      if (T.predictor == GEO_PRED_VAR_TEAM && !T.positivity) {
-        constexpr int ZB = Team<P>::ZB;
-        const unsigned grid = static_cast<unsigned>((T.Z + ZB - 1) / ZB);
-        k_ader_vt<P, R><<<grid, ZB * Dim<P>::N, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
+      if (T.predictor == GEO_PRED_VAR_TEAM && (!T.positivity || RingCfg<P, R>::POS)) {
+        using L = RingLayout<P, R>;
+        const unsigned grid = static_cast<unsigned>((T.Z + L::ZB - 1) / L::ZB);
+        if constexpr (RingCfg<P, R>::POS) {
+          if (T.positivity) {
+            k_ader_ring<P, R, true><<<grid, L::NT, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
+            break;
+          }
+        }
+        k_ader_ring<P, R, false><<<grid, L::NT, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
       } else if (T.predictor != GEO_PRED_ZONE_THREAD) {
         constexpr int ZB = Team<P>::ZB;
         const unsigned grid = static_cast<unsigned>((T.Z + ZB - 1) / ZB);

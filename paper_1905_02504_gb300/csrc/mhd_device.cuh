@@ -312,6 +312,18 @@ __device__ __forceinline__ void st8(double* p, const double* u) {
   for (int c = 0; c < 4; ++c) reinterpret_cast<double2*>(p)[c] = make_double2(u[2 * c], u[2 * c + 1]);
 }
 
+// column and shell of zone z (32-bit division where the index allows it)
+__device__ __forceinline__ void zone_column(long long z, int nr, int& c, int& k) {
+  if ((z >> 32) == 0) {
+    const unsigned q = static_cast<unsigned>(z) / static_cast<unsigned>(nr);
+    c = static_cast<int>(q);
+    k = static_cast<int>(static_cast<unsigned>(z) - q * static_cast<unsigned>(nr));
+  } else {
+    c = static_cast<int>(z / nr);
+    k = static_cast<int>(z % nr);
+  }
+}
+
 __device__ __forceinline__ int side_of_lf(int lf) { return lf == 0 ? 3 : (lf == 1 ? 1 : (lf == 2 ? 0 : 2)); }
 
 template <int P>

@@ -123,7 +123,7 @@ def edge_nodes(p):
     return out
 
 
-# Row groups per (zone, variable) of the variable team: a thread computes the rows
+# Row groups per (zone, variable) of the sparse-row contraction: a thread computes the rows
 # of its group, so fewer groups reuse each loaded 16-byte chunk of F for more
 # rows (FP32 FMAs per chunk: about 8 with 4 groups at p = 4, 15 with 2; the
 # GB300 SM issues 128 FP32 FMAs per 128 B of shared-memory bandwidth, i.e. 16 per
