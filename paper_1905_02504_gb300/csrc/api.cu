@@ -196,7 +196,24 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   D.wE = m->upload(T.wE, err);
   D.st_n = m->upload(T.st_n, err);
   D.st_nb = m->upload(T.st_nb, err);
-  D.pinvH = m->upload(T.pinvH, err);
+  // the fit matrices by stencil zone and the smoothness form's triangle (BulkTables)
+  const int nc1p = (d.NC1 + 3) / 4 * 4;
+  int qtri = 0;
+  for (int i = 0; i < d.NC1; ++i) qtri += (d.NC1 - i + 3) / 4 * 4;
+  std::vector<double> PTt(static_cast<size_t>(T.ncol) * d.SMAX * nc1p, 0.0), Qst(static_cast<size_t>(T.ncol) * qtri, 0.0);
+  for (int c = 0; c < T.ncol; ++c) {
+    for (int j = 0; j < d.SMAX; ++j)
+      for (int i = 0; i < d.NC1; ++i)
+        PTt[(static_cast<size_t>(c) * d.SMAX + j) * nc1p + i] = T.pinvH[(static_cast<size_t>(c) * d.NC1 + i) * d.SMAX + j];
+    size_t at = static_cast<size_t>(c) * qtri;
+    for (int i = 0; i < d.NC1; ++i) {
+      const double* Qc = &T.Q[static_cast<size_t>(c) * d.NC1 * d.NC1];
+      for (int j = i; j < d.NC1; ++j) Qst[at + j - i] = i == j ? Qc[i * d.NC1 + i] : Qc[i * d.NC1 + j] + Qc[j * d.NC1 + i];
+      at += (d.NC1 - i + 3) / 4 * 4;
+    }
+  }
+  D.pinvH = m->upload(PTt, err);
+  D.Qs = nullptr;  // FP32 only
   D.oct_nb = m->upload(T.oct_nb, err);
   D.oct_inv = m->upload(T.oct_inv, err);
   D.Q = m->upload(T.Q, err);
@@ -264,7 +281,7 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   std::vector<double> iJF(T.JF.size()), iJE(T.JE.size());
   for (size_t t = 0; t < iJF.size(); ++t) iJF[t] = 1.0 / T.JF[t];
   for (size_t t = 0; t < iJE.size(); ++t) iJE[t] = 1.0 / T.JE[t];
-  D.b64 = geo::BulkTables<double>{D.pinvH, D.oct_inv, D.Q,        D.TF,       D.nF,       D.wF,
+  D.b64 = geo::BulkTables<double>{D.pinvH, D.oct_inv, D.Q,        D.Qs,      D.TF,       D.nF,       D.wF,
                                   D.GB,    D.GM,      D.TN,      D.J0,       D.iJ0,      D.Sm,       D.gcl,
                                   D.JF,    D.JE,      D.se_t,     D.se_nang,  D.se_nradL, D.se_nradR,
                                   D.sv_fn, D.sv_t,    m->upload(weta, err), m->upload(iJF, err),
@@ -272,12 +289,13 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   const bool f32 = prec == GEO_FP32_BULK;
   if (f32) {
     geo::BulkTables<float>& b = D.b32;
-    b.pinvH = m->upload_f32(T.pinvH, err);
+    b.pinvH = m->upload_f32(PTt, err);
+    b.Qs = m->upload_f32(Qst, err);
     b.oct_inv = m->upload_f32(T.oct_inv, err);
     b.weta = m->upload_f32(weta, err);
     b.iJF = m->upload_f32(iJF, err);
     b.iJE = m->upload_f32(iJE, err);
-    b.Q = m->upload_f32(T.Q, err);
+    b.Q = nullptr;  // the full form is read by the FP64 reverse sweep only
     b.TF = m->upload_f32(T.TF, err);
     b.nF = m->upload_f32(T.nF, err);
     b.wF = m->upload_f32(T.wF, err);

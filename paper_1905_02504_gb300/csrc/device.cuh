@@ -7,15 +7,15 @@ namespace geo {
 
 template <int P> struct Dim;
 template <> struct Dim<2> {
-  static constexpr int N = 8, M = 2, NC1 = 3, NC = 4, NB = 7, NQR = 4, NQS = 4, NQT = 24, NS = 1,
+  static constexpr int N = 8, M = 2, NC1 = 3, NC1P = 4, QTRI = 12, NC = 4, NB = 7, NQR = 4, NQS = 4, NQT = 24, NS = 1,
                        SMAX = 6, NBIN = 3 * NC + NQT + 6, NNZ = 16, NFN = 4, NEN = 2, RL = 2;
 };
 template <> struct Dim<3> {
-  static constexpr int N = 20, M = 3, NC1 = 9, NC = 10, NB = 16, NQR = 4, NQS = 4, NQT = 24, NS = 2,
+  static constexpr int N = 20, M = 3, NC1 = 9, NC1P = 12, QTRI = 60, NC = 10, NB = 16, NQR = 4, NQS = 4, NQT = 24, NS = 2,
                        SMAX = 26, NBIN = 3 * NC + NQT + 6, NNZ = 96, NFN = 8, NEN = 3, RL = 8;
 };
 template <> struct Dim<4> {
-  static constexpr int N = 32, M = 4, NC1 = 19, NC = 20, NB = 30, NQR = 9, NQS = 6, NQT = 42, NS = 3,
+  static constexpr int N = 32, M = 4, NC1 = 19, NC1P = 20, QTRI = 220, NC = 20, NB = 30, NQR = 9, NQS = 6, NQT = 42, NS = 3,
                        SMAX = 32, NBIN = 3 * NC + NQT + 6, NNZ = 192, NFN = 12, NEN = 4, RL = 8;
 };
 
@@ -49,7 +49,10 @@ template <int P, typename R> struct RefConst {
 // [ncol][NBIN][3N], [ncol][3][NBIN] and [ncol][NC1][N], so that the
 // threads of a node team read consecutive entries.
 template <typename R> struct BulkTables {
-  const R *pinvH, *oct_inv, *Q, *TF, *nF, *wF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
+  // pinvH: [ncol][SMAX][NC1P] (coefficients of one stencil zone adjacent, padded to
+  // 16-byte vectors); Qs: upper triangle of Q by rows, off-diagonals doubled, each row
+  // padded to a multiple of 4 entries
+  const R *pinvH, *oct_inv, *Q, *Qs, *TF, *nF, *wF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
   // edge geometry: unit tangents and face normals at the edge points
   const R *se_t, *se_nang, *se_nradL, *se_nradR, *sv_fn, *sv_t;
   // [ncol] (l_0 / |x_0|)^2 of the column's zones (the same along a self-similar
@@ -76,7 +79,7 @@ struct DevTables {
   const int* st_nb;
   const double* pinvH;
   const int* oct_nb;
-  const double *oct_inv, *Q, *V0, *l0, *S0, *A0, *TF, *nF, *wF, *WF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
+  const double *oct_inv, *Q, *Qs, *V0, *l0, *S0, *A0, *TF, *nF, *wF, *WF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
   const int *col_side_se, *col_side_sgn;
   const int *se_v, *se_col, *se_lf, *se_perm, *se_le, *se_rev;
   const double *se_t, *se_dlw, *se_nang, *se_nradL, *se_nradR;

@@ -50,112 +50,230 @@ namespace {
 using namespace dev;
 
 // ----------------------------------------------------------------------------
-// a1: WENO-AO reconstruction (Sec. III); one thread per zone and conserved
-// variable (grid row y = variable)
+// a1: WENO-AO reconstruction (Sec. III); one thread per zone and VB conserved
+// variables (grid row y = group of variables)
+//
+// All lanes of a column read the same matrix entries, and a broadcast costs the L1
+// as much as any other warp-wide word, so in FP32 one variable per thread is bound by
+// those loads (one per multiply-add).  With VB variables an entry loaded once serves
+// VB multiply-adds (p = 4, 147,456 zones: 275 -> 138 us with VB = 4, 145 us with 2;
+// p = 3, 193,536 zones: 172 -> 93 / 100 us; p = 2, 1,327,104 zones: 474 -> 304 / 279 us).
+// In FP32 beta_H comes from the upper triangle of the smoothness form (off-diagonals
+// doubled, rows padded to whole 16-byte vectors).  Both forms take the six face
+// neighbours' differences once for the eight octants that share them.  The FP64 form is
+// bound by its own pipe and keeps VB = 1, which spreads small meshes over more warps;
+// it sums in the order of the reverse sweep's own evaluation (k_adj_weno), bit for bit,
+// so that ties (MinMod between mirror images of a symmetric field) fall to the same side
+// as ever (p = 4, 110,592 zones: 2.02 -> 1.99 ms; a triangular beta_H would give 1.70 ms
+// and turned such ties over).
 // ----------------------------------------------------------------------------
-template <int P, typename R>
-__global__ void __launch_bounds__(TPB) k_weno(const DevTables T, const double* __restrict__ U,
+template <int P> struct WenoVb { static constexpr int VB = P == 2 ? 2 : 4; };
+// zones from which the grid with VB variables per thread still fills the GPU
+constexpr long long WENO_WIDE = 20000;
+
+template <int P, typename R, int VB>
+__global__ void __launch_bounds__(TPB, 3) k_weno(const DevTables T, const double* __restrict__ U,
                                               const float* __restrict__ Uhl, R* __restrict__ Wc) {
   using Dm = Dim<P>;
-  constexpr int NC1 = Dm::NC1, SMAX = Dm::SMAX;
+  constexpr int NC1 = Dm::NC1, NC1P = Dm::NC1P, SMAX = Dm::SMAX, CH = 16 / sizeof(R);
   const R GH = R(0.85), GK = R(0.15 / 8.0), EPS0 = R(1e-12);
-  long long z = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const long long z = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (z >= T.Z) return;
   const BulkTables<R>& B = bulk<R>(T);
   const long long Z = T.Z;
-  int nr = T.nr;
-  int c = static_cast<int>(z / nr), k = static_cast<int>(z % nr);
-  int ns = T.st_n[c];
-  long long zs[SMAX];
-  for (int j = 0; j < ns; ++j) {
-    int pk = T.st_nb[c * SMAX + j];
-    int cc = pk >> 3, dk = (pk & 7) - 3;
-    int kk = min(max(k + dk, 0), nr - 1);
-    zs[j] = static_cast<long long>(cc) * nr + kk;
-  }
-  long long zo[24];
+  const int nr = T.nr, v0 = blockIdx.y * VB;
+  int c, k;
+  zone_column(z, nr, c, k);
+  auto zone_of = [&](int pk) {
+    return static_cast<long long>(pk >> 3) * nr + min(max(k + (pk & 7) - 3, 0), nr - 1);
+  };
+  // zone-average differences U_j - U_0: in FP64 for the FP64 form; in the
+  // FP32-bulk form from the hi/lo split, (hi_j - hi_0) + (lo_j - lo_0), which
+  // carries the FP64 difference to FP32 rounding without FP64 arithmetic
+  R u0[VB], l0[VB], EPS[VB];
+  const R weta = B.weta[c];
 #pragma unroll
-  for (int j = 0; j < 24; ++j) {
-    int pk = T.oct_nb[c * 24 + j];
-    int cc = pk >> 3, dk = (pk & 7) - 3;
-    int kk = min(max(k + dk, 0), nr - 1);
-    zo[j] = static_cast<long long>(cc) * nr + kk;
-  }
-  const R* pinv = B.pinvH + static_cast<size_t>(c) * NC1 * SMAX;
-  const R* oinv = B.oct_inv + static_cast<size_t>(c) * 72;
-  const R* Qm = B.Q + static_cast<size_t>(c) * NC1 * NC1;
-  {
-    const int v = blockIdx.y;  // one conserved variable per grid row
-    const double* Uv = U + v * Z;
-    // zone-average differences U_j - U_0: in FP64 for the FP64 form; in the
-    // FP32-bulk form from the hi/lo split, (hi_j - hi_0) + (lo_j - lo_0), which
-    // carries the FP64 difference to FP32 rounding without FP64 arithmetic
-    const float* Hv = Uhl ? Uhl + static_cast<size_t>(v) * Z : nullptr;
-    const float* Lv = Uhl ? Uhl + static_cast<size_t>(8 + v) * Z : nullptr;
-    const double u0d = (sizeof(R) == 8) ? Uv[z] : 0.0;
-    const float h0 = (sizeof(R) == 4) ? Hv[z] : 0.f, l0 = (sizeof(R) == 4) ? Lv[z] : 0.f;
-    // eps = eps_0 + K (l_0/r_0)^2 u_0^2 with K = 1 (Arandiga et al. 2011: eps ~ h^2)
-    const R u0 = (sizeof(R) == 8) ? static_cast<R>(u0d) : static_cast<R>(h0);
-    const R EPS = EPS0 + B.weta[c] * u0 * u0;
-    auto diff = [&](long long zz) -> R {
-      if constexpr (sizeof(R) == 4) return (Hv[zz] - h0) + (Lv[zz] - l0);
-      else return static_cast<R>(Uv[zz] - u0d);
-    };
-    R uH[NC1];
-#pragma unroll
-    for (int m = 0; m < NC1; ++m) uH[m] = R(0);
-    for (int j = 0; j < ns; ++j) {
-      R du = diff(zs[j]);
-#pragma unroll
-      for (int m = 0; m < NC1; ++m) uH[m] += pinv[m * SMAX + j] * du;
+  for (int v = 0; v < VB; ++v) {
+    const size_t at = static_cast<size_t>(v0 + v) * Z + z;
+    if constexpr (sizeof(R) == 4) {
+      u0[v] = Uhl[at];
+      l0[v] = Uhl[8 * Z + at];
+    } else {
+      u0[v] = U[at];
+      l0[v] = R(0);
     }
-    R bH = R(0);
+    // eps = eps_0 + K (l_0/r_0)^2 u_0^2 with K = 1 (Arandiga et al. 2011: eps ~ h^2)
+    EPS[v] = EPS0 + weta * u0[v] * u0[v];
+  }
+  auto diff = [&](int v, long long zz) -> R {
+    const size_t at = static_cast<size_t>(v0 + v) * Z + zz;
+    if constexpr (sizeof(R) == 4) return (Uhl[at] - u0[v]) + (Uhl[8 * Z + at] - l0[v]);
+    else return U[at] - u0[v];
+  };
+  // ---- central fit
+  R uH[VB][NC1];
+#pragma unroll
+  for (int v = 0; v < VB; ++v)
+#pragma unroll
+    for (int m = 0; m < NC1; ++m) uH[v][m] = R(0);
+  {
+    const int ns = T.st_n[c];
+    const int* nb = T.st_nb + c * SMAX;
+    const R* pinv = B.pinvH + static_cast<size_t>(c) * SMAX * NC1P;
+#pragma unroll 2
+    for (int j = 0; j < ns; ++j) {
+      const long long zz = zone_of(nb[j]);
+      R du[VB], a[NC1P];
+#pragma unroll
+      for (int v = 0; v < VB; ++v) du[v] = diff(v, zz);
+#pragma unroll
+      for (int t = 0; t < NC1P / CH; ++t) ld16(pinv + j * NC1P + t * CH, a + t * CH);
+#pragma unroll
+      for (int v = 0; v < VB; ++v)
+#pragma unroll
+        for (int m = 0; m < NC1; ++m) uH[v][m] += a[m] * du[v];
+    }
+  }
+  // ---- beta_H = uH^T Q uH
+  R bH[VB];
+#pragma unroll
+  for (int v = 0; v < VB; ++v) bH[v] = R(0);
+  if constexpr (sizeof(R) == 4) {
+    const R* q = B.Qs + static_cast<size_t>(c) * Dm::QTRI;
+#pragma unroll
+    for (int i = 0; i < NC1; ++i) {
+      R row[NC1P];
+      const int n = NC1 - i, np = (n + 3) / 4 * 4;
+#pragma unroll
+      for (int t = 0; t < NC1P / CH; ++t)
+        if (t * CH < np) ld16(q + t * CH, row + t * CH);
+      q += np;
+#pragma unroll
+      for (int v = 0; v < VB; ++v) {
+        R s = row[0] * uH[v][i];
+#pragma unroll
+        for (int j = 1; j < n; ++j) s += row[j] * uH[v][i + j];
+        bH[v] += uH[v][i] * s;
+      }
+    }
+  } else {
+    const R* Qm = B.Q + static_cast<size_t>(c) * NC1 * NC1;
 #pragma unroll
     for (int i = 0; i < NC1; ++i) {
       R s = R(0);
 #pragma unroll
-      for (int j = 0; j < NC1; ++j) s += Qm[i * NC1 + j] * uH[j];
-      bH += uH[i] * s;
+      for (int j = 0; j < NC1; ++j) s += Qm[i * NC1 + j] * uH[0][j];
+      bH[0] += uH[0][i] * s;
     }
-    R uK[8][3], wK[8];
-    R tau = R(0);
+  }
+  // ---- octant fits from the differences of the six face neighbours: octant o takes
+  // neighbours 0/1, 2/3, 4/5 by the bits of o
+  R d6[VB][6];
 #pragma unroll
-    for (int o = 0; o < 8; ++o) {
-      R d0 = diff(zo[3 * o]), d1 = diff(zo[3 * o + 1]), d2 = diff(zo[3 * o + 2]);
-      const R* A = oinv + 9 * o;
+  for (int f = 0; f < 6; ++f) {
+    const int o = (f & 1) << (f >> 1);  // an octant that holds neighbour f
+    const long long zz = zone_of(T.oct_nb[c * 24 + 3 * o + (f >> 1)]);
 #pragma unroll
-      for (int a = 0; a < 3; ++a) uK[o][a] = A[3 * a] * d0 + A[3 * a + 1] * d1 + A[3 * a + 2] * d2;
-      wK[o] = uK[o][0] * uK[o][0] + uK[o][1] * uK[o][1] + uK[o][2] * uK[o][2];  // beta_k for now
-      tau += fabs(bH - wK[o]);
+    for (int v = 0; v < VB; ++v) d6[v][f] = diff(v, zz);
+  }
+  const R* oinv = B.oct_inv + static_cast<size_t>(c) * 72;
+  auto octant = [&](int o, const R* A, const R* d, R* u) {
+    const R d0 = d[o & 1], d1 = d[2 + ((o >> 1) & 1)], d2 = d[4 + ((o >> 2) & 1)];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) u[a] = A[3 * a] * d0 + A[3 * a + 1] * d1 + A[3 * a + 2] * d2;
+  };
+  constexpr bool KEEP = VB == 1;  // keep the octant gradients (else form them twice)
+  R wK[VB][8], tau[VB], uK[1][8][3];
+#pragma unroll
+  for (int v = 0; v < VB; ++v) tau[v] = R(0);
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    R A[9];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) A[t] = oinv[9 * o + t];
+#pragma unroll
+    for (int v = 0; v < VB; ++v) {
+      R u[3];
+      octant(o, A, d6[v], u);
+      wK[v][o] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];  // beta_k for now
+      tau[v] += fabs(bH[v] - wK[v][o]);
+      if constexpr (KEEP) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) uK[0][o][a] = u[a];
+      }
     }
-    // WENO-Z type weights g (1 + (tau / (beta + eps))^2), tau = mean |beta_H - beta_k|
-    // (Borges, Carmona, Costa & Don 2008), with the mesh-dependent eps above
-    tau *= R(0.125);
-    const R rH = tau / (bH + EPS);
+  }
+  // ---- WENO-Z type weights g (1 + (tau / (beta + eps))^2), tau = mean |beta_H - beta_k|
+  // (Borges, Carmona, Costa & Don 2008), with the mesh-dependent eps above
+  R fH[VB];
+#pragma unroll
+  for (int v = 0; v < VB; ++v) {
+    tau[v] *= R(0.125);
+    const R rH = tau[v] / (bH[v] + EPS[v]);
     R wH = GH * (R(1) + rH * rH);
     R tot = wH;
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
-      const R r = tau / (wK[o] + EPS);
-      wK[o] = GK * (R(1) + r * r);
-      tot += wK[o];
+      const R r = tau[v] / (wK[v][o] + EPS[v]);
+      wK[v][o] = GK * (R(1) + r * r);
+      tot += wK[v][o];
     }
-    R itot = R(1) / tot;
+    const R itot = R(1) / tot;
     wH *= itot;
-    R fH = wH / GH;
-    R* out = Wc + static_cast<size_t>(v) * NC1 * Z;
+    fH[v] = wH / GH;
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      if constexpr (sizeof(R) == 4) wK[v][o] = wK[v][o] * itot - fH[v] * GK;
+      else wK[v][o] *= itot;
+    }
+  }
+  // out_a = fH (uH_a - GK sum_o uK_oa) + sum_o w_o uK_oa (a < 3), out_m = fH uH_m
+  R s3[VB][3];
+  if constexpr (sizeof(R) == 8) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       R sk = R(0), wk = R(0);
 #pragma unroll
       for (int o = 0; o < 8; ++o) {
-        sk += uK[o][a];
-        wk += wK[o] * itot * uK[o][a];
+        sk += uK[0][o][a];
+        wk += wK[0][o] * uK[0][o][a];
       }
-      out[a * Z + z] = fH * (uH[a] - GK * sk) + wk;
+      s3[0][a] = fH[0] * (uH[0][a] - GK * sk) + wk;
     }
+  } else {
+    // with the octants' net weights w_o - fH GK
 #pragma unroll
-    for (int m = 3; m < NC1; ++m) out[m * Z + z] = fH * uH[m];
+    for (int v = 0; v < VB; ++v)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) s3[v][a] = fH[v] * uH[v][a];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      R A[9];
+      if constexpr (!KEEP) {
+#pragma unroll
+        for (int t = 0; t < 9; ++t) A[t] = oinv[9 * o + t];
+      }
+#pragma unroll
+      for (int v = 0; v < VB; ++v) {
+        R u[3];
+        if constexpr (KEEP) {
+#pragma unroll
+          for (int a = 0; a < 3; ++a) u[a] = uK[0][o][a];
+        } else {
+          octant(o, A, d6[v], u);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) s3[v][a] += wK[v][o] * u[a];
+      }
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < VB; ++v) {
+    R* out = Wc + static_cast<size_t>(v0 + v) * NC1 * Z + z;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) out[a * Z] = s3[v][a];
+#pragma unroll
+    for (int m = 3; m < NC1; ++m) out[m * Z] = fH[v] * uH[v][m];
   }
 }
 
@@ -531,27 +649,6 @@ template <> struct Team<4> { static constexpr int ZB = 4; };
 // access phase, handle the same node (P = 2, 3) or two nodes (P = 4) of several
 // zones; the per-zone stride XS is padded to 1 (2) modulo the 8 bank groups so
 // that those zones' copies of one chunk sit in distinct bank groups.
-template <typename R> struct Chunk { static constexpr int CH = 16 / sizeof(R), NCH = 8 / CH; };
-
-template <typename R>
-__device__ __forceinline__ void ld16(const R* p, R* out) {
-  if constexpr (sizeof(R) == 4) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
-    out[0] = q.x; out[1] = q.y; out[2] = q.z; out[3] = q.w;
-  } else {
-    const double2 q = *reinterpret_cast<const double2*>(p);
-    out[0] = q.x; out[1] = q.y;
-  }
-}
-template <typename R>
-__device__ __forceinline__ void st16(R* p, const R* in) {
-  if constexpr (sizeof(R) == 4) {
-    *reinterpret_cast<float4*>(p) = make_float4(in[0], in[1], in[2], in[3]);
-  } else {
-    *reinterpret_cast<double2*>(p) = make_double2(in[0], in[1]);
-  }
-}
-
 template <int P, typename R>
 struct TeamSmem {
   using Dm = Dim<P>;
@@ -1584,7 +1681,14 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
   R* trE = static_cast<R*>(S.trE);
   switch (stage) {
     case ST_WENO:
-      k_weno<P, R><<<dim3(grid_for(T.Z), 8), TPB, 0, st>>>(T, S.U, sizeof(R) == 4 ? S.Uhl : nullptr, Wc);
+      if constexpr (sizeof(R) == 4) {
+        if (T.Z >= WENO_WIDE) {
+          constexpr int VB = WenoVb<P>::VB;
+          k_weno<P, R, VB><<<dim3(grid_for(T.Z), 8 / VB), TPB, 0, st>>>(T, S.U, S.Uhl, Wc);
+          break;
+        }
+      }
+      k_weno<P, R, 1><<<dim3(grid_for(T.Z), 8), TPB, 0, st>>>(T, S.U, S.Uhl, Wc);
       break;
     case ST_BPERP:
       k_bperp<P, R><<<grid_for(T.F), TPB, 0, st>>>(T, S.U, S.phi, Wc, Bp);

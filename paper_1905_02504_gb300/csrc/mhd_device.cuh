@@ -289,6 +289,28 @@ __device__ __forceinline__ size_t trE_at(long long z, int m, int idx, long long 
   return (static_cast<size_t>((m - 1) * 12 * Dim<P>::NS + idx) * Z + z) * 8;
 }
 
+// 16-byte vectors of the bulk type
+template <typename R> struct Chunk { static constexpr int CH = 16 / sizeof(R), NCH = 8 / CH; };
+
+template <typename R>
+__device__ __forceinline__ void ld16(const R* p, R* out) {
+  if constexpr (sizeof(R) == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    out[0] = q.x; out[1] = q.y; out[2] = q.z; out[3] = q.w;
+  } else {
+    const double2 q = *reinterpret_cast<const double2*>(p);
+    out[0] = q.x; out[1] = q.y;
+  }
+}
+template <typename R>
+__device__ __forceinline__ void st16(R* p, const R* in) {
+  if constexpr (sizeof(R) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(in[0], in[1], in[2], in[3]);
+  } else {
+    *reinterpret_cast<double2*>(p) = make_double2(in[0], in[1]);
+  }
+}
+
 // 16-byte loads and stores of an 8-value state (16-byte aligned)
 __device__ __forceinline__ void ld8(const float* p, float* u) {
   const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
