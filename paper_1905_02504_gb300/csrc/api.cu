@@ -271,6 +271,53 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   D.sv_fn = m->upload(T.sv_fn, err);
   D.sv_t = m->upload(T.sv_t, err);
   D.sv_dlw = m->upload(T.sv_dlw, err);
+  // radial edges in ring order, with each face's normal turned to point from its first
+  // to its second ring zone
+  const int NS = d.NS, M1 = d.M - 1;
+  std::vector<int> rcol(static_cast<size_t>(T.nsv) * 4), rle(rcol.size());
+  std::vector<double> rfn(static_cast<size_t>(T.nsv) * 4 * NS * 3, 0.0);
+  for (int sv = 0; sv < T.nsv && err == cudaSuccess; ++sv) {
+    const int nz = T.sv_nc[sv];
+    const int* fL = &T.sv_fL[4 * sv];
+    const int* fR = &T.sv_fR[4 * sv];
+    int at = 0;
+    bool used[4] = {false, false, false, false};
+    for (int j = 0; j < nz; ++j) {
+      rcol[4 * sv + j] = T.sv_col[4 * sv + at];
+      rle[4 * sv + j] = T.sv_le[4 * sv + at];
+      int f = -1;
+      for (int t = 0; t < nz && f < 0; ++t)
+        if (!used[t] && (fL[t] == at || fR[t] == at)) f = t;
+      if (f < 0) {
+        err = cudaErrorInvalidValue;
+        break;
+      }
+      used[f] = true;
+      const double sg = fL[f] == at ? 1.0 : -1.0;
+      for (int t = 0; t < NS * 3; ++t)
+        rfn[(static_cast<size_t>(4) * sv + j) * NS * 3 + t] = sg * T.sv_fn[(static_cast<size_t>(4) * sv + f) * NS * 3 + t];
+      at = fL[f] == at ? fR[f] : fL[f];
+    }
+    if (at != 0) err = cudaErrorInvalidValue;  // the ring must close
+    for (int j = nz; j < 4; ++j) {
+      rcol[4 * sv + j] = rcol[4 * sv];
+      rle[4 * sv + j] = rle[4 * sv];
+    }
+  }
+  D.svr_col = m->upload(rcol, err);
+  D.svr_le = m->upload(rle, err);
+  // Gauss weights times point weights
+  std::vector<double> WFt(static_cast<size_t>(T.ncol) * M1 * d.NQT), sew(static_cast<size_t>(T.nse) * M1 * NS),
+      svw(static_cast<size_t>(T.nsv) * M1 * NS);
+  auto times = [&](std::vector<double>& out, const std::vector<double>& w, int rows, int n) {
+    for (int r = 0; r < rows; ++r)
+      for (int k = 0; k < M1; ++k)
+        for (int t = 0; t < n; ++t)
+          out[(static_cast<size_t>(r) * M1 + k) * n + t] = T.wt[k] * w[static_cast<size_t>(r) * n + t];
+  };
+  times(WFt, T.WF, T.ncol, d.NQT);
+  times(sew, T.se_dlw, T.nse, NS);
+  times(svw, T.sv_dlw, T.nsv, NS);
   // (l_0 / |x_0|)^2 per column: the WENO-AO eps scale
   std::vector<double> weta(T.ncol);
   for (int c = 0; c < T.ncol; ++c) {
@@ -284,8 +331,8 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   D.b64 = geo::BulkTables<double>{D.pinvH, D.oct_inv, D.Q,        D.Qs,      D.TF,       D.nF,       D.wF,
                                   D.GB,    D.GM,      D.TN,      D.J0,       D.iJ0,      D.Sm,       D.gcl,
                                   D.JF,    D.JE,      D.se_t,     D.se_nang,  D.se_nradL, D.se_nradR,
-                                  D.sv_fn, D.sv_t,    m->upload(weta, err), m->upload(iJF, err),
-                                  m->upload(iJE, err)};
+                                  m->upload(rfn, err), D.sv_t, m->upload(WFt, err), m->upload(sew, err), m->upload(svw, err),
+                                  m->upload(weta, err), m->upload(iJF, err), m->upload(iJE, err)};
   const bool f32 = prec == GEO_FP32_BULK;
   if (f32) {
     geo::BulkTables<float>& b = D.b32;
@@ -312,7 +359,10 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
     b.se_nang = m->upload_f32(T.se_nang, err);
     b.se_nradL = m->upload_f32(T.se_nradL, err);
     b.se_nradR = m->upload_f32(T.se_nradR, err);
-    b.sv_fn = m->upload_f32(T.sv_fn, err);
+    b.svr_fn = m->upload_f32(rfn, err);
+    b.WFt = m->upload_f32(WFt, err);
+    b.se_w = m->upload_f32(sew, err);
+    b.sv_w = m->upload_f32(svw, err);
     b.sv_t = m->upload_f32(T.sv_t, err);
   }
   if (err == cudaSuccess) {

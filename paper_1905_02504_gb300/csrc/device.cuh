@@ -53,8 +53,12 @@ template <typename R> struct BulkTables {
   // 16-byte vectors); Qs: upper triangle of Q by rows, off-diagonals doubled, each row
   // padded to a multiple of 4 entries
   const R *pinvH, *oct_inv, *Q, *Qs, *TF, *nF, *wF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
-  // edge geometry: unit tangents and face normals at the edge points
-  const R *se_t, *se_nang, *se_nradL, *se_nradR, *sv_fn, *sv_t;
+  // edge geometry: unit tangents and face normals at the edge points (around a radial
+  // edge in ring order, svr_fn [nsv][4][NS][3])
+  const R *se_t, *se_nang, *se_nradL, *se_nradR, *svr_fn, *sv_t;
+  // Gauss weight times point weight: [ncol][M-1][NQT] of the face points, [nse][M-1][NS]
+  // and [nsv][M-1][NS] of the edge points (times |dl|), at shell 0
+  const R *WFt, *se_w, *sv_w;
   // [ncol] (l_0 / |x_0|)^2 of the column's zones (the same along a self-similar
   // column): the mesh scale of the WENO-AO eps, eps = 1e-12 + weta u_0^2
   const R* weta;
@@ -85,6 +89,9 @@ struct DevTables {
   const double *se_t, *se_dlw, *se_nang, *se_nradL, *se_nradR;
   const int *sv_nc, *sv_col, *sv_le, *sv_fL, *sv_fR, *sv_fse;
   const double *sv_fn, *sv_t, *sv_dlw;
+  // zones around a radial edge in ring order (face j between zones j and j + 1; three
+  // zones: the fourth entry repeats the first): column, local edge [nsv][4]
+  const int *svr_col, *svr_le;
   BulkTables<double> b64;
   BulkTables<float> b32;
 };

@@ -1098,177 +1098,224 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
 #include "ader_ring.cuh"
 
 // ----------------------------------------------------------------------------
-// a4: face fluxes (HLL at face points x Gauss times, FP64 accumulation)
+// a4: face fluxes (HLL or HLLD at face points x Gauss times)
+//
+// SPLIT threads (1 or 4 neighbouring lanes) per face take its points in turn and add
+// up their sums.  The FP64 pipe needs 64 cycles of an SM quarter for one instruction
+// of a warp, so a mesh with fewer faces than FACE_SPLIT_MAX, whose warps do not fill
+// the 608 quarters, is as slow as one thread's points in a row; four threads a face
+// cut that chain by four (162 zones at p = 3: 76 -> 24 us), and cost the sums of eight
+// variables over two shuffle steps where the chip is full.
+// The quadrature weight times the Gauss weight is tabulated in the bulk type; the
+// shell's factor q^2k enters once, in FP64.
 // ----------------------------------------------------------------------------
-template <int P, typename R, bool HLLD>
+constexpr long long FACE_SPLIT_MAX = 40000;
+
+// sum of x over the S neighbouring lanes of a group, in all of them
+template <int S, typename R>
+__device__ __forceinline__ R lane_sum(R x) {
+#pragma unroll
+  for (int o = 1; o < S; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+template <int P, typename R, bool HLLD, int SPLIT>
 __global__ void __launch_bounds__(TPB) k_face_flux(const DevTables T, const R* __restrict__ trF,
                                                    double* __restrict__ Ff, double dt) {
   using Dm = Dim<P>;
   constexpr int M = Dm::M, NQT = Dm::NQT;
-  long long f = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (f >= T.F) return;
+  const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const long long F = T.F, Z = T.Z;
+  const long long f = t / SPLIT < F ? t / SPLIT : F - 1;
   const BulkTables<R>& BT = bulk<R>(T);
-  const long long Z = T.Z, F = T.F;
-  FaceInfo fi = face_info(T, f);
-  int nq = nq_of<P>(fi.lfg);
-  double s2 = T.qpow[fi.k] * T.qpow[fi.k];
+  const FaceInfo fi = face_info(T, f);
+  const int nq = nq_of<P>(fi.lfg);
   const R gs = static_cast<R>(fi.gsign);
   const R g = static_cast<R>(T.gamma);
+  const R* W = BT.WFt + static_cast<size_t>(fi.cg) * (M - 1) * NQT + foff<P>(fi.lfg);
+  const R* nF = BT.nF + (static_cast<size_t>(fi.cg) * NQT + foff<P>(fi.lfg)) * 3;
   // quadrature sum over the face's points and Gauss times in the bulk type (the
   // zone update that sums the faces is FP64)
   R acc[8];
 #pragma unroll
   for (int v = 0; v < 8; ++v) acc[v] = R(0);
+  int m = 1, q = SPLIT == 1 ? 0 : static_cast<int>(t % SPLIT);
 #pragma unroll 1
-  for (int m = 1; m < M; ++m) {
-    double wt = T.wt[m - 1];
-#pragma unroll 1
-    for (int q = 0; q < nq; ++q) {
-      int ig = foff<P>(fi.lfg) + q;
-      const R* nv = BT.nF + (static_cast<size_t>(fi.cg) * NQT + ig) * 3;
-      R nx = gs * nv[0], ny = gs * nv[1], nz = gs * nv[2];
-      const R W = static_cast<R>(wt * T.WF[static_cast<size_t>(fi.cg) * NQT + ig] * s2);
-      R uL[8], uR[8];
-      if (fi.zL >= 0) ld8(trF + trF_at<P>(fi.zL, m, foff<P>(fi.lfL) + q, Z), uL);
-      if (fi.zR >= 0) {
-        int ql = q;
-        if (fi.se >= 0) ql = T.se_perm[fi.se * Dm::NQS + q];
-        ld8(trF + trF_at<P>(fi.zR, m, foff<P>(fi.lfR) + ql, Z), uR);
-      }
-      if (fi.zL < 0) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) uL[v] = uR[v];
-      }
-      if (fi.zR < 0) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) uR[v] = uL[v];
-      }
-      if constexpr (HLLD) hlld_acc(uL, uR, nx, ny, nz, g, W, acc);
-      else hll_acc(uL, uR, nx, ny, nz, g, W, acc);
+  while (true) {
+    while (q >= nq) {
+      q -= nq;
+      ++m;
     }
-  }
+    if (m >= M) break;
+    const R* nv = nF + 3 * q;
+    const R nx = gs * nv[0], ny = gs * nv[1], nz = gs * nv[2];
+    const R w = W[(m - 1) * NQT + q];
+    R uL[8], uR[8];
+    if (fi.zL >= 0) ld8(trF + trF_at<P>(fi.zL, m, foff<P>(fi.lfL) + q, Z), uL);
+    if (fi.zR >= 0) {
+      const int ql = fi.se >= 0 ? T.se_perm[fi.se * Dm::NQS + q] : q;
+      ld8(trF + trF_at<P>(fi.zR, m, foff<P>(fi.lfR) + ql, Z), uR);
+    }
+    if (fi.zL < 0) {
 #pragma unroll
-  for (int v = 0; v < 8; ++v) Ff[v * F + f] = dt * static_cast<double>(acc[v]);
+      for (int v = 0; v < 8; ++v) uL[v] = uR[v];
+    }
+    if (fi.zR < 0) {
+#pragma unroll
+      for (int v = 0; v < 8; ++v) uR[v] = uL[v];
+    }
+    if constexpr (HLLD) hlld_acc(uL, uR, nx, ny, nz, g, w, acc);
+    else hll_acc(uL, uR, nx, ny, nz, g, w, acc);
+    q += SPLIT;
+  }
+  const double s2 = dt * (T.qpow[fi.k] * T.qpow[fi.k]);
+#pragma unroll
+  for (int v = 0; v < 8; ++v) {
+    const R a = lane_sum<SPLIT>(acc[v]);
+    if (t < F * SPLIT && (SPLIT == 1 || t % SPLIT == v % SPLIT)) Ff[v * F + f] = s2 * static_cast<double>(a);
+  }
 }
 
 // ----------------------------------------------------------------------------
-// a5: edge EMFs (multidimensional Rusanov at edge points x Gauss times, FP64
-// accumulation)
+// a5: edge EMFs (multidimensional Rusanov at edge points x Gauss times)
+//
+// The zones around an edge are walked as a ring: face j lies between zones j and
+// j + 1 (three zones at a cube corner: the ring closes on a copy of zone 0; two at a
+// boundary edge: one face).  Every index is then static, each zone's sound and Alfven
+// speeds are formed once for its two faces, and no state has to be picked by a runtime
+// index (before: 16 three-way selects per face and point).  SPLIT threads per edge
+// share its points on meshes of fewer than EDGE_SPLIT_MAX edges, as for the faces (162
+// zones at p = 3: 84 -> 25 us).  FP32 p = 4, 147,456 zones: 257 -> 182 us; FP64 p = 4,
+// 110,592 zones: 2.66 -> 2.44 ms.
 // ----------------------------------------------------------------------------
-template <int P, typename R>
+constexpr long long EDGE_SPLIT_MAX = 40000;
+
+template <int P, typename R, int SPLIT>
 __global__ void __launch_bounds__(TPB) k_edge_emf(const DevTables T, const R* __restrict__ trE,
                                                   double* __restrict__ Ee, double dt) {
   using Dm = Dim<P>;
-  constexpr int M = Dm::M, NS = Dm::NS;
-  long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= T.E) return;
-  const long long Z = T.Z;
+  constexpr int M = Dm::M, NS = Dm::NS, NP = (M - 1) * NS;
+  const long long t0 = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const long long E = T.E, Z = T.Z;
+  const long long e = t0 / SPLIT < E ? t0 / SPLIT : E - 1;
   const int nr = T.nr;
   const R g = static_cast<R>(T.gamma);
-  long long zs[4];
-  int les[4], revs[4];
-  int nz = 0, nf = 0;
-  int fL[4], fR[4];
   const BulkTables<R>& BT = bulk<R>(T);
-  const R* fn[4];  // normals [NS][3] of each face
-  R tv[NS][3], dlw[NS];
+  long long zs[4];
+  int le[4];          // first edge point of the zone's local edge, or the last one if reversed
+  int rev = 0;        // bit j: zone j counts the points from the other end
+  int nz, nf;         // zones and faces around the edge
+  const R* fn[4];     // normals [NS][3] of the ring's faces
+  R fs[4] = {R(1), R(1), R(1), R(1)};  // their sign
+  const R *tv, *tw;   // tangents (one for a radial edge), weights [M-1][NS]
+  int ts;             // stride of the tangents
+  double q;
   if (e < T.E_rad) {
-    int sv = static_cast<int>(e / nr), k = static_cast<int>(e % nr);
+    int sv, k;
+    zone_column(e, nr, sv, k);
     nz = T.sv_nc[sv];
     nf = nz;
-    for (int j = 0; j < nz; ++j) {
-      zs[j] = static_cast<long long>(T.sv_col[4 * sv + j]) * nr + k;
-      les[j] = T.sv_le[4 * sv + j];
-      revs[j] = 0;
-      fL[j] = T.sv_fL[4 * sv + j];
-      fR[j] = T.sv_fR[4 * sv + j];
-      fn[j] = BT.sv_fn + static_cast<size_t>(sv * 4 + j) * NS * 3;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      zs[j] = static_cast<long long>(T.svr_col[4 * sv + j]) * nr + k;
+      le[j] = T.svr_le[4 * sv + j] * NS;
+      fn[j] = BT.svr_fn + static_cast<size_t>(sv * 4 + j) * NS * 3;
     }
-    for (int s = 0; s < NS; ++s) {
-      for (int a = 0; a < 3; ++a) tv[s][a] = BT.sv_t[3 * sv + a];
-      dlw[s] = static_cast<R>(T.sv_dlw[sv * NS + s] * T.qpow[k]);
-    }
+    tv = BT.sv_t + 3 * sv;
+    ts = 0;
+    tw = BT.sv_w + static_cast<size_t>(sv) * NP;
+    q = T.qpow[k];
   } else {
-    long long r = e - T.E_rad;
-    int se = static_cast<int>(r / (nr + 1)), kk = static_cast<int>(r % (nr + 1));
-    int cL = T.se_col[2 * se], cR = T.se_col[2 * se + 1];
-    int revL = T.se_rev[2 * se], revR = T.se_rev[2 * se + 1];
+    int se, kk;
+    zone_column(e - T.E_rad, nr + 1, se, kk);
+    const int cL = T.se_col[2 * se], cR = T.se_col[2 * se + 1];
+    const int rL = T.se_rev[2 * se], rR = T.se_rev[2 * se + 1];
     const R* nang = BT.se_nang + static_cast<size_t>(se) * NS * 3;
     if (kk >= 1 && kk <= nr - 1) {
-      nz = 4;
-      zs[0] = static_cast<long long>(cL) * nr + kk - 1; les[0] = T.se_le[(2 * se) * 2 + 1]; revs[0] = revL;
-      zs[1] = static_cast<long long>(cL) * nr + kk;     les[1] = T.se_le[(2 * se) * 2 + 0]; revs[1] = revL;
-      zs[2] = static_cast<long long>(cR) * nr + kk - 1; les[2] = T.se_le[(2 * se + 1) * 2 + 1]; revs[2] = revR;
-      zs[3] = static_cast<long long>(cR) * nr + kk;     les[3] = T.se_le[(2 * se + 1) * 2 + 0]; revs[3] = revR;
-      nf = 4;
-      fL[0] = 0; fR[0] = 2; fn[0] = nang;
-      fL[1] = 1; fR[1] = 3; fn[1] = nang;
-      fL[2] = 0; fR[2] = 1; fn[2] = BT.se_nradL + static_cast<size_t>(se) * NS * 3;
-      fL[3] = 2; fR[3] = 3; fn[3] = BT.se_nradR + static_cast<size_t>(se) * NS * 3;
+      // ring: L below, L above, R above, R below
+      nz = nf = 4;
+      zs[0] = static_cast<long long>(cL) * nr + kk - 1; le[0] = T.se_le[4 * se + 1];
+      zs[1] = zs[0] + 1;                                le[1] = T.se_le[4 * se];
+      zs[3] = static_cast<long long>(cR) * nr + kk - 1; le[3] = T.se_le[4 * se + 3];
+      zs[2] = zs[3] + 1;                                le[2] = T.se_le[4 * se + 2];
+      rev = (rL ? 3 : 0) | (rR ? 12 : 0);
+      fn[0] = BT.se_nradL + static_cast<size_t>(se) * NS * 3;
+      fn[1] = fn[3] = nang;
+      fn[2] = BT.se_nradR + static_cast<size_t>(se) * NS * 3;
+      fs[2] = fs[3] = R(-1);
     } else {
       nz = 2;
-      int top = (kk == nr) ? 1 : 0;
-      int kz = top ? nr - 1 : 0;
-      zs[0] = static_cast<long long>(cL) * nr + kz; les[0] = T.se_le[(2 * se) * 2 + top]; revs[0] = revL;
-      zs[1] = static_cast<long long>(cR) * nr + kz; les[1] = T.se_le[(2 * se + 1) * 2 + top]; revs[1] = revR;
       nf = 1;
-      fL[0] = 0; fR[0] = 1; fn[0] = nang;
+      const int top = kk == nr ? 1 : 0, kz = top ? nr - 1 : 0;
+      zs[0] = static_cast<long long>(cL) * nr + kz; le[0] = T.se_le[4 * se + top];
+      zs[1] = static_cast<long long>(cR) * nr + kz; le[1] = T.se_le[4 * se + 2 + top];
+      zs[2] = zs[3] = zs[0];
+      le[2] = le[3] = le[0];
+      rev = (rL ? 1 : 0) | (rR ? 2 : 0);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) fn[j] = nang;
     }
-    for (int s = 0; s < NS; ++s) {
-      for (int a = 0; a < 3; ++a) tv[s][a] = BT.se_t[(static_cast<size_t>(se) * NS + s) * 3 + a];
-      dlw[s] = static_cast<R>(T.se_dlw[se * NS + s] * T.qpow[kk]);
-    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) le[j] *= NS;
+    tv = BT.se_t + static_cast<size_t>(se) * NS * 3;
+    ts = 3;
+    tw = BT.se_w + static_cast<size_t>(se) * NP;
+    q = T.qpow[kk];
   }
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if ((rev >> j) & 1) le[j] += NS - 1;
   const R inz = R(1) / static_cast<R>(nz);
   R acc = R(0);  // quadrature sum in the bulk type; the Phi update is FP64
 #pragma unroll 1
-  for (int m = 1; m < M; ++m) {
-    const R wt = static_cast<R>(T.wt[m - 1]);
-#pragma unroll 1
-    for (int s = 0; s < NS; ++s) {
-      // primitive state of each zone at the point, 1/rho formed once per zone
-      // (register arrays: every index below is static or goes through sel4)
-      R ir[4], vx[4], vy[4], vz[4], pr[4], bx[4], by[4], bz[4];
+  for (int pt = SPLIT == 1 ? 0 : static_cast<int>(t0 % SPLIT); pt < NP; pt += SPLIT) {
+    const int m = pt / NS + 1, s = pt % NS;
+    const R tx = tv[ts * s], ty = tv[ts * s + 1], tz = tv[ts * s + 2];
+    // per zone: v, B, s = a^2 + b^2 and 4 a^2 / rho of the fast speed (1/rho formed once)
+    R vx[4], vy[4], vz[4], bx[4], by[4], bz[4], sq[4], qa[4];
+    R Ev = R(0);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        R u[8] = {R(1), R(0), R(0), R(0), R(1), R(0), R(0), R(0)};
-        if (j < nz) {
-          const int sl = revs[j] ? NS - 1 - s : s;
-          ld8(trE + trE_at<P>(zs[j], m, les[j] * NS + sl, Z), u);
-        }
-        const Prim<R> w = to_prim(u, g);
-        ir[j] = R(1) / u[0];
-        vx[j] = w.vx; vy[j] = w.vy; vz[j] = w.vz; pr[j] = w.p;
-        bx[j] = w.bx; by[j] = w.by; bz[j] = w.bz;
+    for (int j = 0; j < 4; ++j) {
+      if (j >= nz) {  // the ring closes: zone 0 again (three zones); unused otherwise
+        vx[j] = vx[0]; vy[j] = vy[0]; vz[j] = vz[0];
+        bx[j] = bx[0]; by[j] = by[0]; bz[j] = bz[0];
+        sq[j] = sq[0]; qa[j] = qa[0];
+        continue;
       }
-      R tx = tv[s][0], ty = tv[s][1], tz = tv[s][2];
-      R E = R(0);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        // (-v x B) . t
-        if (j < nz)
-          E -= (vy[j] * bz[j] - vz[j] * by[j]) * tx + (vz[j] * bx[j] - vx[j] * bz[j]) * ty +
-               (vx[j] * by[j] - vy[j] * bx[j]) * tz;
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j >= nf) continue;
-        const R* nvd = fn[j] + 3 * s;
-        R nx = nvd[0], ny = nvd[1], nzz = nvd[2];
-        const int qL = fL[j], qR = fR[j];
-        R a = fmax(rusanov_speed_ir(sel4(ir, qL), sel4(vx, qL), sel4(vy, qL), sel4(vz, qL), sel4(pr, qL),
-                                    sel4(bx, qL), sel4(by, qL), sel4(bz, qL), nx, ny, nzz, g),
-                   rusanov_speed_ir(sel4(ir, qR), sel4(vx, qR), sel4(vy, qR), sel4(vz, qR), sel4(pr, qR),
-                                    sel4(bx, qR), sel4(by, qR), sel4(bz, qR), nx, ny, nzz, g));
-        // t x n
-        R cx = ty * nzz - tz * ny, cy = tz * nx - tx * nzz, cz = tx * ny - ty * nx;
-        R dbx = sel4(bx, qR) - sel4(bx, qL), dby = sel4(by, qR) - sel4(by, qL), dbz = sel4(bz, qR) - sel4(bz, qL);
-        E += a * (dbx * cx + dby * cy + dbz * cz);
-      }
-      acc += wt * dlw[s] * (E * inz);
+      R u[8];
+      ld8(trE + trE_at<P>(zs[j], m, le[j] + (((rev >> j) & 1) ? -s : s), Z), u);
+      const R ir = R(1) / u[0];
+      vx[j] = u[1] * ir; vy[j] = u[2] * ir; vz[j] = u[3] * ir;
+      bx[j] = u[5]; by[j] = u[6]; bz[j] = u[7];
+      const R hb = R(0.5) * (bx[j] * bx[j] + by[j] * by[j] + bz[j] * bz[j]);
+      const R p = (g - R(1)) * ((u[4] - hb) - R(0.5) * (u[1] * vx[j] + u[2] * vy[j] + u[3] * vz[j]));
+      const R a2 = g * p * ir;
+      sq[j] = a2 + R(2) * hb * ir;
+      qa[j] = R(4) * a2 * ir;
+      // (-v x B) . t
+      Ev -= (vy[j] * bz[j] - vz[j] * by[j]) * tx + (vz[j] * bx[j] - vx[j] * bz[j]) * ty +
+            (vx[j] * by[j] - vy[j] * bx[j]) * tz;
     }
+    auto speed = [&](int j, R nx, R ny, R nzz) {
+      const R bn = bx[j] * nx + by[j] * ny + bz[j] * nzz;
+      return fabs(vx[j] * nx + vy[j] * ny + vz[j] * nzz) +
+             sqrt(R(0.5) * (sq[j] + sqrt(fmax(sq[j] * sq[j] - qa[j] * (bn * bn), R(0)))));
+    };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j >= nf) continue;
+      const int r = (j + 1) & 3;
+      const R* nv = fn[j] + 3 * s;
+      const R nx = nv[0], ny = nv[1], nzz = nv[2];
+      const R a = fs[j] * fmax(speed(j, nx, ny, nzz), speed(r, nx, ny, nzz));
+      // a (B_r - B_j) . (t x n)
+      Ev += a * ((bx[r] - bx[j]) * (ty * nzz - tz * ny) + (by[r] - by[j]) * (tz * nx - tx * nzz) +
+                 (bz[r] - bz[j]) * (tx * ny - ty * nx));
+    }
+    acc += tw[pt] * (Ev * inz);
   }
-  Ee[e] = dt * static_cast<double>(acc);
+  acc = lane_sum<SPLIT>(acc);
+  if (t0 < E * SPLIT && (SPLIT == 1 || t0 % SPLIT == 0)) Ee[e] = dt * q * static_cast<double>(acc);
 }
 
 // ----------------------------------------------------------------------------
@@ -1718,14 +1765,22 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
         k_ader<P, R, false><<<grid_for(T.Z), TPB, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
       }
       break;
-    case ST_FACE:
-      if (T.riemann == GEO_RIEMANN_HLLD)
-        k_face_flux<P, R, true><<<grid_for(T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
-      else
-        k_face_flux<P, R, false><<<grid_for(T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
+    case ST_FACE: {
+      auto run = [&](auto hlld) {
+        if (T.F <= FACE_SPLIT_MAX)
+          k_face_flux<P, R, hlld.value, 4><<<grid_for(4 * T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
+        else
+          k_face_flux<P, R, hlld.value, 1><<<grid_for(T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
+      };
+      if (T.riemann == GEO_RIEMANN_HLLD) run(std::true_type{});
+      else run(std::false_type{});
       break;
+    }
     case ST_EDGE:
-      k_edge_emf<P, R><<<grid_for(T.E), TPB, 0, st>>>(T, trE, S.Ee, dt);
+      if (P > 2 && T.E <= EDGE_SPLIT_MAX)
+        k_edge_emf<P, R, P == 2 ? 1 : 4><<<grid_for(4 * T.E), TPB, 0, st>>>(T, trE, S.Ee, dt);
+      else
+        k_edge_emf<P, R, 1><<<grid_for(T.E), TPB, 0, st>>>(T, trE, S.Ee, dt);
       break;
     case ST_UPD_U:
       k_update_u<<<grid_for(T.Z), TPB, 0, st>>>(T, S.U, S.Ff, S.Uhl);

@@ -66,30 +66,70 @@ __device__ __forceinline__ R fast_speed(const Prim<R>& w, R nx, R ny, R nz, R g)
   return sqrt(R(0.5) * (s + sqrt(fmax(s * s - R(4) * a2 * bn2, R(0)))));
 }
 
-// HLL flux along the unit normal (Davis wave speeds); the weighted flux is
-// accumulated in the type A
-template <typename R, typename A>
-__device__ __forceinline__ void hll_acc(const R* uL, const R* uR, R nx, R ny, R nz, R g, A w, A* acc) {
-  Prim<R> a = to_prim(uL, g), b = to_prim(uR, g);
-  R vnL = a.vx * nx + a.vy * ny + a.vz * nz;
-  R vnR = b.vx * nx + b.vy * ny + b.vz * nz;
-  R cL = fast_speed(a, nx, ny, nz, g), cR = fast_speed(b, nx, ny, nz, g);
-  R SL = fmin(vnL - cL, vnR - cR);
-  R SR = fmax(vnL + cL, vnR + cR);
-  R FL[8], FR[8];
-  flux_n(uL, a, nx, ny, nz, FL);
-  flux_n(uR, b, nx, ny, nz, FR);
+// One side of a face for the HLL flux along the unit normal n: normal velocity and
+// field, total pressure, total enthalpy, v.B and the fast speed, 1/rho formed once.
+template <typename R>
+struct HllSide {
+  R vx, vy, vz, vn, bn, pt, H, vb, c;
+};
+template <typename R>
+__device__ __forceinline__ HllSide<R> hll_side(const R* u, R nx, R ny, R nz, R g) {
+  HllSide<R> a;
+  const R ir = R(1) / u[0];
+  a.vx = u[1] * ir;
+  a.vy = u[2] * ir;
+  a.vz = u[3] * ir;
+  const R hb = R(0.5) * (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]);
+  const R p = (g - R(1)) * ((u[4] - hb) - R(0.5) * (u[1] * a.vx + u[2] * a.vy + u[3] * a.vz));
+  a.pt = p + hb;
+  a.H = u[4] + a.pt;
+  a.vn = a.vx * nx + a.vy * ny + a.vz * nz;
+  a.bn = u[5] * nx + u[6] * ny + u[7] * nz;
+  a.vb = a.vx * u[5] + a.vy * u[6] + a.vz * u[7];
+  const R a2 = g * p * ir, s = a2 + R(2) * hb * ir, bn2 = a.bn * a.bn * ir;
+  a.c = sqrt(R(0.5) * (s + sqrt(fmax(s * s - R(4) * a2 * bn2, R(0)))));
+  return a;
+}
+// acc += w F(u).n from one side's quantities
+template <typename R>
+__device__ __forceinline__ void hll_one_side(const R* u, const HllSide<R>& a, R nx, R ny, R nz, R w, R* acc) {
+  const R wv = w * a.vn, wb = w * a.bn, wp = w * a.pt;
+  acc[0] += u[0] * wv;
+  acc[1] += u[1] * wv - u[5] * wb + wp * nx;
+  acc[2] += u[2] * wv - u[6] * wb + wp * ny;
+  acc[3] += u[3] * wv - u[7] * wb + wp * nz;
+  acc[4] += a.H * wv - a.vb * wb;
+  acc[5] += u[5] * wv - a.vx * wb;
+  acc[6] += u[6] * wv - a.vy * wb;
+  acc[7] += u[7] * wv - a.vz * wb;
+}
+
+// acc += w times the HLL flux along the unit normal (Davis wave speeds).  With
+// a = w S_R / (S_R - S_L), b = -w S_L / (S_R - S_L) and d = a S_L it is
+// a F_L + b F_R + d (U_R - U_L), formed from a v_n, a B_n, ... directly: about 200 FP64
+// operations a point against 245 with both fluxes written out and combined (p = 4,
+// 110,592 zones: 2.79 -> 2.58 ms).
+template <typename R>
+__device__ __forceinline__ void hll_acc(const R* uL, const R* uR, R nx, R ny, R nz, R g, R w, R* acc) {
+  const HllSide<R> l = hll_side(uL, nx, ny, nz, g), r = hll_side(uR, nx, ny, nz, g);
+  const R SL = fmin(l.vn - l.c, r.vn - r.c);
+  const R SR = fmax(l.vn + l.c, r.vn + r.c);
   if (SL >= R(0)) {
-#pragma unroll
-    for (int v = 0; v < 8; ++v) acc[v] += w * static_cast<A>(FL[v]);
+    hll_one_side(uL, l, nx, ny, nz, w, acc);
   } else if (SR <= R(0)) {
-#pragma unroll
-    for (int v = 0; v < 8; ++v) acc[v] += w * static_cast<A>(FR[v]);
+    hll_one_side(uR, r, nx, ny, nz, w, acc);
   } else {
-    R id = R(1) / (SR - SL);
-#pragma unroll
-    for (int v = 0; v < 8; ++v)
-      acc[v] += w * static_cast<A>((SR * FL[v] - SL * FR[v] + SL * SR * (uR[v] - uL[v])) * id);
+    const R wi = w * (R(1) / (SR - SL));
+    const R a = wi * SR, b = -(wi * SL), d = a * SL;
+    const R av = a * l.vn, ab = a * l.bn, bv = b * r.vn, bb = b * r.bn, p = a * l.pt + b * r.pt;
+    acc[0] += av * uL[0] + bv * uR[0] + d * (uR[0] - uL[0]);
+    acc[1] += av * uL[1] - ab * uL[5] + bv * uR[1] - bb * uR[5] + p * nx + d * (uR[1] - uL[1]);
+    acc[2] += av * uL[2] - ab * uL[6] + bv * uR[2] - bb * uR[6] + p * ny + d * (uR[2] - uL[2]);
+    acc[3] += av * uL[3] - ab * uL[7] + bv * uR[3] - bb * uR[7] + p * nz + d * (uR[3] - uL[3]);
+    acc[4] += av * l.H - ab * l.vb + bv * r.H - bb * r.vb + d * (uR[4] - uL[4]);
+    acc[5] += av * uL[5] - ab * l.vx + bv * uR[5] - bb * r.vx + d * (uR[5] - uL[5]);
+    acc[6] += av * uL[6] - ab * l.vy + bv * uR[6] - bb * r.vy + d * (uR[6] - uL[6]);
+    acc[7] += av * uL[7] - ab * l.vz + bv * uR[7] - bb * r.vz + d * (uR[7] - uL[7]);
   }
 }
 
@@ -222,24 +262,6 @@ template <typename R>
 __device__ __forceinline__ R rusanov_speed(const R* u, R nx, R ny, R nz, R g) {
   Prim<R> w = to_prim(u, g);
   return fabs(w.vx * nx + w.vy * ny + w.vz * nz) + fast_speed(w, nx, ny, nz, g);
-}
-
-// the same Rusanov speed from a primitive state whose 1/rho is already formed
-template <typename R>
-__device__ __forceinline__ R rusanov_speed_ir(R ir, R vx, R vy, R vz, R p, R bx, R by, R bz, R nx, R ny, R nz,
-                                              R g) {
-  R a2 = g * p * ir;
-  R b2 = (bx * bx + by * by + bz * bz) * ir;
-  R bn = bx * nx + by * ny + bz * nz;
-  R bn2 = bn * bn * ir;
-  R s = a2 + b2;
-  return fabs(vx * nx + vy * ny + vz * nz) + sqrt(R(0.5) * (s + sqrt(fmax(s * s - R(4) * a2 * bn2, R(0)))));
-}
-
-// a[q] for a runtime q in 0..3 of a register array (selects, no local memory)
-template <typename T>
-__device__ __forceinline__ T sel4(const T (&a)[4], int q) {
-  return q == 0 ? a[0] : (q == 1 ? a[1] : (q == 2 ? a[2] : a[3]));
 }
 
 template <typename R>
