@@ -381,10 +381,11 @@ __device__ __forceinline__ int nq_of(int lf) {
 }
 
 // face f -> L zone / local face, R zone / local face (-1 when on the boundary),
-// the column and local face whose tables hold the face geometry, shell index k
+// the zones' columns, the column and local face whose tables hold the face geometry,
+// shell index k
 struct FaceInfo {
   long long zL, zR;
-  int lfL, lfR, cg, lfg, k, se;
+  int lfL, lfR, cL, cR, cg, lfg, k, se;
   double gsign;  // canonical normal = gsign * outward normal of (cg, lfg)
 };
 
@@ -392,8 +393,9 @@ __device__ __forceinline__ FaceInfo face_info(const DevTables& T, long long f) {
   FaceInfo fi;
   int nr = T.nr;
   if (f < T.F_rad) {
-    int c = static_cast<int>(f / (nr + 1));
-    int k = static_cast<int>(f % (nr + 1));
+    int c, k;
+    zone_column(f, nr + 1, c, k);
+    fi.cL = fi.cR = c;
     fi.zL = (k >= 1) ? static_cast<long long>(c) * nr + k - 1 : -1;
     fi.zR = (k < nr) ? static_cast<long long>(c) * nr + k : -1;
     fi.lfL = 5;
@@ -404,10 +406,11 @@ __device__ __forceinline__ FaceInfo face_info(const DevTables& T, long long f) {
     fi.k = k;
     fi.se = -1;
   } else {
-    long long r = f - T.F_rad;
-    int se = static_cast<int>(r / nr);
-    int k = static_cast<int>(r % nr);
-    int cL = T.se_col[2 * se], cR = T.se_col[2 * se + 1];
+    int se, k;
+    zone_column(f - T.F_rad, nr, se, k);
+    const int cL = T.se_col[2 * se], cR = T.se_col[2 * se + 1];
+    fi.cL = cL;
+    fi.cR = cR;
     fi.zL = static_cast<long long>(cL) * nr + k;
     fi.zR = static_cast<long long>(cR) * nr + k;
     fi.lfL = T.se_lf[2 * se];
