@@ -269,8 +269,7 @@ int geo_probe_contraction(geo_mesh_t mesh, int tensor, int64_t zones, int reps, 
  * the nodes, Uh_dev [M][8][N][zones] the result (J times the conserved state at
  * node i and time level tau_m: tau_1 = 0, then the Gauss points).  Node order as
  * geo_prism_nodes.  Enqueued on `stream` (0 = legacy default), no
- * synchronisation; the reference tables (< 20 KB per order) are built and copied
- * to the device on the first call of each order and kept until exit.
+ * synchronisation and no device memory of its own.
  * GEO_ERR_ARG for a bad order, zone count, null pointer, dt <= 0 or gamma <= 1. */
 int geo_prism_predictor(int order, int64_t zones, const double* X_dev, const double* U_dev, double dt, double gamma,
                         double* Uh_dev, void* stream);

@@ -4,7 +4,6 @@
 #include <cmath>
 #include <cstring>
 #include <memory>
-#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -937,67 +936,6 @@ int geo_probe_fma_peak(int prec, void* stream, double* flops_per_s) {
   return GEO_OK;
 }
 
-// prism tables per order on the device, built on first use and kept until exit
-namespace {
-struct PrismTables {
-  std::once_flag once;
-  int status = GEO_ERR_CUDA;
-  std::string err;
-  int N = 0;
-  std::vector<double> nodes;
-  double* Dv = nullptr;         // [3][N][RL] nonzeros of each row of D^alpha
-  unsigned char* Dc = nullptr;  // [3][N][RL] their columns (padding: value 0, the row's own column)
-  double* R = nullptr;          // [M][M]
-};
-PrismTables g_prism[3];
-
-PrismTables& prism_tables_for(int p) {
-  PrismTables& P = g_prism[p - 2];
-  std::call_once(P.once, [&]() {
-    std::vector<double> D, wt, R;
-    if (!geo::prism_element(p, P.nodes, D)) {
-      P.status = GEO_ERR_ARG;
-      P.err = "prism element: singular basis";
-      return;
-    }
-    geo::time_tables(p, wt, R);
-    const int N = static_cast<int>(P.nodes.size() / 3), RL = geo::prism_rl(p);
-    P.N = N;
-    std::vector<double> Dv(static_cast<size_t>(3) * N * RL, 0.0);
-    std::vector<unsigned char> Dc(static_cast<size_t>(3) * N * RL, 0);
-    for (int a = 0; a < 3; ++a)
-      for (int i = 0; i < N; ++i) {
-        int r = 0;
-        for (int j = 0; j < N; ++j) {
-          const double d = D[(static_cast<size_t>(a) * N + i) * N + j];
-          if (d == 0.0) continue;
-          if (r == RL) {
-            P.status = GEO_ERR_ARG;
-            P.err = "prism element: a row of D has more nonzeros than the row form holds";
-            return;
-          }
-          Dv[(static_cast<size_t>(a) * N + i) * RL + r] = d;
-          Dc[(static_cast<size_t>(a) * N + i) * RL + r] = static_cast<unsigned char>(j);
-          ++r;
-        }
-        for (; r < RL; ++r) Dc[(static_cast<size_t>(a) * N + i) * RL + r] = static_cast<unsigned char>(i);
-      }
-    cudaError_t e = cudaMalloc(&P.Dv, Dv.size() * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&P.Dc, Dc.size());
-    if (e == cudaSuccess) e = cudaMalloc(&P.R, R.size() * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemcpy(P.Dv, Dv.data(), Dv.size() * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(P.Dc, Dc.data(), Dc.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(P.R, R.data(), R.size() * sizeof(double), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      P.err = std::string("prism tables: ") + cudaGetErrorString(e);
-      return;
-    }
-    P.status = GEO_OK;
-  });
-  return P;
-}
-}  // namespace
-
 int geo_prism_nodes(int order, double* nodes, int64_t count) {
   if (order < 2 || order > 4 || !nodes) return fail(GEO_ERR_ARG, "geo_prism_nodes: bad arguments");
   std::vector<double> n, D;
@@ -1029,9 +967,9 @@ int geo_prism_predictor(int order, int64_t zones, const double* X_dev, const dou
                         double* Uh_dev, void* stream) {
   if (order < 2 || order > 4 || zones < 1 || !X_dev || !U_dev || !Uh_dev || !(dt > 0.0) || !(gamma > 1.0))
     return fail(GEO_ERR_ARG, "geo_prism_predictor: bad arguments");
-  PrismTables& P = prism_tables_for(order);
-  if (P.status != GEO_OK) return fail(P.status, P.err);
-  cudaError_t e = geo::launch_prism_predictor_any(order, zones, P.Dv, P.Dc, P.R, X_dev, U_dev, dt, gamma, Uh_dev,
+  std::vector<double> wt, R;
+  geo::time_tables(order, wt, R);
+  cudaError_t e = geo::launch_prism_predictor_any(order, zones, R.data(), X_dev, U_dev, dt, gamma, Uh_dev,
                                                   static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "geo_prism_predictor");
   return GEO_OK;

@@ -6,7 +6,9 @@ flux differences of Eqs. C.34 / D.29 in nodal collocation form), and the nodes o
 each face and edge of the reference cube (the supports of the point
 evaluations at face and edge points).  Only the pattern is compiled in; the
 values still come from the host tables at mesh creation, which check that every
-nonzero of their D^alpha lies in this pattern.
+nonzero of their D^alpha lies in this pattern.  And, for the prism predictor, the
+derivative matrices of the triangular Lagrange element of degree p-1 along its
+edges 0-1 and 0-2, entries and exact values.
 
 The element is the one the host tables build: the unit cube [-1/2, 1/2]^3, the
 monomials of superlinear degree <= p-1, nodes = the 8 vertices
@@ -152,6 +154,47 @@ def row_groups(p, pat):
     return rg
 
 
+def triangle_nodes(p):
+    """Nodes of a prism's triangular face in the prism's node order, as coordinates
+    (s, t) of the oblique frame vertex 0 + s (v1 - v0) + t (v2 - v0): the vertices,
+    p - 2 equidistant nodes inside the sides 0-1, 1-2, 2-0, at p = 4 the centroid."""
+    v = [(Fr(0), Fr(0)), (Fr(1), Fr(0)), (Fr(0), Fr(1))]
+    out = list(v)
+    for a, b in ((0, 1), (1, 2), (2, 0)):
+        for k in range(1, p - 1):
+            f = Fr(k, p - 1)
+            out.append(tuple((1 - f) * v[a][d] + f * v[b][d] for d in range(2)))
+    if p == 4:
+        out.append((Fr(1, 3), Fr(1, 3)))
+    return out
+
+
+def triangle_derivatives(p):
+    """[direction] -> list of (i, j, value) of the nonzero derivatives at node i of the
+    basis function of node j, by row then column."""
+    xs = triangle_nodes(p)
+    ex = [(a, d - a) for d in range(p) for a in range(d, -1, -1)]
+    n = len(xs)
+    assert n == len(ex)
+    C = _inverse([[x[0] ** a * x[1] ** b for a, b in ex] for x in xs])
+    out = []
+    for ax in range(2):
+        ent = []
+        for i, x in enumerate(xs):
+            dm = []
+            for e in ex:
+                if e[ax] == 0:
+                    dm.append(Fr(0))
+                else:
+                    dm.append(e[ax] * x[ax] ** (e[ax] - 1) * x[1 - ax] ** e[1 - ax])
+            for j in range(n):
+                d = sum(dm[m] * C[m][j] for m in range(n))
+                if d != 0:
+                    ent.append((i, j, d))
+        out.append(ent)
+    return out
+
+
 def header():
     lines = ["// Generated by paper_1905_02504_gb300/refpattern.py at build time; do not edit.",
              "// Nonzero pattern of the nodal derivative matrices D^alpha and the face / edge",
@@ -176,6 +219,20 @@ def header():
         lines.append("  static constexpr int G = %d;" % (len(rg) - 1))
         lines.append("  static constexpr int RG[%d] = {%s};" % (len(rg), ", ".join(map(str, rg))))
         lines.append("  static constexpr int EG[3][%d] = {%s};" % (len(rg), ", ".join("{%s}" % ", ".join(map(str, e)) for e in eg)))
+        lines.append("};")
+    lines.append("// derivatives of the triangular element along its edges 0-1 and 0-2")
+    lines.append("template <int P> struct TriPattern;")
+    for p in (2, 3, 4):
+        ent = triangle_derivatives(p)
+        nnz = len(ent[0])
+        assert len(ent[1]) == nnz
+        flat = [e for ax in ent for e in ax]
+        lines.append("template <> struct TriPattern<%d> {" % p)
+        lines.append("  static constexpr int NNZ = %d;" % nnz)
+        lines.append("  static constexpr unsigned char I[%d] = {%s};" % (len(flat), ", ".join(str(e[0]) for e in flat)))
+        lines.append("  static constexpr unsigned char J[%d] = {%s};" % (len(flat), ", ".join(str(e[1]) for e in flat)))
+        lines.append("  static constexpr double V[%d] = {%s};" % (
+            len(flat), ", ".join("%d.0 / %d.0" % (e[2].numerator, e[2].denominator) for e in flat)))
         lines.append("};")
     lines.append("}  // namespace geo")
     return "\n".join(lines) + "\n"
