@@ -330,10 +330,12 @@ __device__ __forceinline__ void ring_points(const R* Fz, int q, const RefConst<P
   }
 }
 
-template <int P, typename R, bool POS>
+// STORE: also write the levels (times J) after each of the first P-1 Picard iterations to
+// itS ([P-1][M-1][8][N][Z]), the linearisation points of the reverse sweep
+template <int P, typename R, bool POS, bool STORE = false>
 __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
     k_ader_ring(const DevTables T, double* __restrict__ U, const double* __restrict__ phi, const R* __restrict__ Wc,
-                const R* __restrict__ Bp, R* __restrict__ trF, R* __restrict__ trE, double dt) {
+                const R* __restrict__ Bp, R* __restrict__ trF, R* __restrict__ trE, double dt, R* __restrict__ itS) {
   using Dm = Dim<P>;
   using L = RingLayout<P, R>;
   using G = Ring<P>;
@@ -688,6 +690,18 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
   // first iteration every level equals level 1, so its flux difference serves all
   const R fs = S.fs[zl] * iJ;
   R base[ML][8], Um[ML][8];
+  const R j0 = valid ? BT.J0[static_cast<size_t>(c) * N + i] : R(1);
+  auto keep = [&](int it) {
+    if constexpr (STORE) {
+      if (valid) {
+#pragma unroll
+        for (int k = 0; k < ML; ++k)
+#pragma unroll
+          for (int v = 0; v < 8; ++v)
+            itS[((static_cast<size_t>(it * ML + k) * 8 + v) * N + i) * Z + z] = j0 * Um[k][v];
+      }
+    }
+  };
   {
     R d0[8];
 #pragma unroll
@@ -703,6 +717,7 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
       }
     }
   }
+  keep(0);
 #pragma unroll 1
   for (int it = 1; it < P; ++it) {
 #pragma unroll
@@ -725,10 +740,10 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
         Um[k][v] = s;
       }
     }
+    if (it < P - 1) keep(it);
   }
   // ---- final levels J U in ring order around the radial axis
   {
-    const R j0 = valid ? BT.J0[static_cast<size_t>(c) * N + i] : R(1);
 #pragma unroll
     for (int m = 0; m < ML; ++m)
 #pragma unroll

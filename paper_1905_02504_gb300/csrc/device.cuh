@@ -142,7 +142,7 @@ cudaError_t upload_reference_constants(const Tables& T);
 // launchers (kernels.cu); return cudaGetLastError() of the launch
 template <int P, typename R>
 cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, double dt, cudaStream_t st);
-// the FP64 node-team predictor (no positivity) that also stores its Picard
+// the FP64 predictor (no positivity) that also stores its Picard
 // iterates for the reverse sweep (It: [P-1][M-1][8][N][Z] doubles)
 template <int P>
 cudaError_t launch_ader_store_iterates(const DevTables& T, const DevState& S, double* It, double dt, cudaStream_t st);

@@ -869,13 +869,11 @@ template <> struct TeamOcc<2, double> { static constexpr int MINB = 4; };
 template <> struct TeamOcc<3, double> { static constexpr int MINB = 2; };
 template <> struct TeamOcc<4, double> { static constexpr int MINB = 2; };
 
-// STORE: also write the levels after each of the first P-1 Picard iterations to
-// itS ([P-1][M-1][8][N][Z]), the linearisation points of the reverse sweep
-template <int P, typename R, bool POS, bool STORE = false>
+template <int P, typename R, bool POS>
 __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
     k_ader_team(const DevTables T, double* __restrict__ U, const double* __restrict__ phi,
                 const R* __restrict__ Wc, const R* __restrict__ Bp, R* __restrict__ trF, R* __restrict__ trE,
-                double dt, R* __restrict__ itS) {
+                double dt) {
   using Dm = Dim<P>;
   constexpr int N = Dm::N, M = Dm::M, NC1 = Dm::NC1, NC = Dm::NC, NQT = Dm::NQT, NS = Dm::NS,
                 NBIN = Dm::NBIN, NR = 3 + 3 * Dm::N, ZB = Team<P>::ZB, NT = ZB * N;
@@ -972,12 +970,6 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
 #pragma unroll
         for (int m = 1; m < M; ++m) s -= rk[m] * dF[m][v];
         Uh[kk][v] = s;
-      }
-      if constexpr (STORE) {
-        if (it < P - 1 && valid) {
-#pragma unroll
-          for (int v = 0; v < 8; ++v) itS[((static_cast<size_t>(it * (M - 1) + kk - 1) * 8 + v) * N + i) * Z + z] = Uh[kk][v];
-        }
       }
     }
   }
@@ -1698,11 +1690,6 @@ cudaError_t upload_reference_constants(const Tables& T) {
           if (!in_pat[al][T.Drow[al * Dm::NNZ + t]][j]) return cudaErrorInvalidValue;
     for (int t = 0; t < 6 * Dm::NFN; ++t)
       if (T.fnode[t] != RP::FN[t]) return cudaErrorInvalidValue;
-    // the node-team reverse predictor holds each column of D^alpha in AdjCols<P>::CL slots
-    for (int al = 0; al < 3; ++al)
-      for (int j = 0; j < Dm::N; ++j)
-        if (T.Dptr[al * (Dm::N + 1) + j + 1] - T.Dptr[al * (Dm::N + 1) + j] > AdjCols<P>::CL)
-          return cudaErrorInvalidValue;
     for (int t = 0; t < 12 * Dm::NEN; ++t)
       if (T.enode[t] != RP::EN[t]) return cudaErrorInvalidValue;
   }
@@ -1753,18 +1740,18 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
         const unsigned grid = static_cast<unsigned>((T.Z + L::ZB - 1) / L::ZB);
         if constexpr (RingCfg<P, R>::POS) {
           if (T.positivity) {
-            k_ader_ring<P, R, true><<<grid, L::NT, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
+            k_ader_ring<P, R, true><<<grid, L::NT, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt, nullptr);
             break;
           }
         }
-        k_ader_ring<P, R, false><<<grid, L::NT, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
+        k_ader_ring<P, R, false><<<grid, L::NT, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt, nullptr);
       } else if (T.predictor != GEO_PRED_ZONE_THREAD) {
         constexpr int ZB = Team<P>::ZB;
         const unsigned grid = static_cast<unsigned>((T.Z + ZB - 1) / ZB);
         if (T.positivity)
-          k_ader_team<P, R, true><<<grid, ZB * Dim<P>::N, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt, nullptr);
+          k_ader_team<P, R, true><<<grid, ZB * Dim<P>::N, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
         else
-          k_ader_team<P, R, false><<<grid, ZB * Dim<P>::N, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt, nullptr);
+          k_ader_team<P, R, false><<<grid, ZB * Dim<P>::N, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
       } else if (T.positivity) {
         k_ader<P, R, true><<<grid_for(T.Z), TPB, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
         k_pos_traces<P, R><<<grid_for(T.Z), TPB, 0, st>>>(T, S.U, trF, trE);
@@ -1838,9 +1825,9 @@ cudaError_t launch_adj_ader(const DevTables& T, const DevState& S, const AdjStat
 
 template <int P>
 cudaError_t launch_ader_store_iterates(const DevTables& T, const DevState& S, double* It, double dt, cudaStream_t st) {
-  constexpr int ZB = Team<P>::ZB;
-  const unsigned grid = static_cast<unsigned>((T.Z + ZB - 1) / ZB);
-  k_ader_team<P, double, false, true><<<grid, ZB * Dim<P>::N, 0, st>>>(
+  using L = RingLayout<P, double>;
+  const unsigned grid = static_cast<unsigned>((T.Z + L::ZB - 1) / L::ZB);
+  k_ader_ring<P, double, false, true><<<grid, L::NT, 0, st>>>(
       T, S.U, S.phi, static_cast<const double*>(S.Wc), static_cast<const double*>(S.Bp), static_cast<double*>(S.trF),
       static_cast<double*>(S.trE), dt, It);
   return cudaGetLastError();
