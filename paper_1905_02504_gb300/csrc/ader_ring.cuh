@@ -348,7 +348,11 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
   const BulkTables<R>& BT = bulk<R>(T);
   const long long Z = T.Z, F = T.F;
   const int nr = T.nr;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // (the warp index through a shuffle, so that the compiler keeps what follows from it,
+  // the point indices and their addresses above all, in uniform registers)
+  // (p = 2, 1,327,104 zones: 917 -> 877 us, p = 3, 193,536: 582 -> 561 us, FP32; at p = 4
+  // it costs registers that are not there: 1288 -> 1462 us)
+  const int tid = threadIdx.x, lane = tid & 31, warp = P == 4 ? tid >> 5 : __shfl_sync(0xffffffffu, tid >> 5, 0);
   const long long zbase = static_cast<long long>(blockIdx.x) * ZB;
   int c0, k0;
   zone_column(zbase, nr, c0, k0);
@@ -644,7 +648,7 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
           const R o = __shfl_xor_sync(0xffffffffu, Fa[v], 1 << a);
-          Gf[v] += up ? Fa[v] - o : o - Fa[v];
+          Gf[v] += (up ? Fa[v] : o) - (up ? o : Fa[v]);  // operands picked, one subtraction
         }
       }
 #pragma unroll
@@ -761,7 +765,8 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
     column(zt, ct, kt);
     const bool in = zbase + zt < Z;
     if (!in) ct = c0;
-    const size_t at = static_cast<size_t>(zbase + zt) * 8 + v;
+    const size_t at = static_cast<size_t>(zbase + (t >> 2) * 4) * 8 + (P == 4 ? lane : 0);
+    const int mine = P == 4 ? 0 : lane;  // the task's 4 x 8 values, one per lane
     const R* iJF = BT.iJF + static_cast<size_t>(ct) * NQT;
     const R* iJE = BT.iJE + static_cast<size_t>(ct) * 12 * Dm::NS;
     // (1/J through the read-only path: the compiler may then keep it across the stores)
@@ -769,7 +774,7 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
       const R w = __ldg(iJ + idx);
       R* o = out + at + static_cast<size_t>(static_cast<unsigned>(idx)) * Z8;
 #pragma unroll
-      for (int m = 0; m < static_cast<int>(sizeof(s) / sizeof(R)); ++m) emit(in, s[m] * w, o + (m0 + m) * step);
+      for (int m = 0; m < static_cast<int>(sizeof(s) / sizeof(R)); ++m) emit(in, s[m] * w, o + (m0 + m) * step + mine);
     };
     const R* row = S.F + zt * L::FL + v * L::RS;
     // all levels together share the weights' and addresses' work; with positivity, whose
