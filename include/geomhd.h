@@ -189,8 +189,8 @@ int geo_cfl_dt(geo_mesh_t mesh, double cfl, double* dt);
  * face fluxes and multidimensional edge EMFs, finite-volume update of U and the
  * Yee constrained-transport update of phi (Eqs. 2.5-2.6).  Asynchronous on the
  * mesh stream.  The U update raises a device flag when a zone leaves rho > 0,
- * p > 0 or is not finite; the flag is copied to pinned host memory after every
- * step, and a later geo_step whose predecessor's copy has landed returns
+ * p > 0 or is not finite; the flag is handed to pinned host memory at the end of
+ * every step, and a later geo_step whose predecessor's copy has landed returns
  * GEO_ERR_NONPHYSICAL without launching anything (the state is left as
  * computed, for inspection).  geo_check_state reads the flag synchronously. */
 int geo_step(geo_mesh_t mesh, double dt);

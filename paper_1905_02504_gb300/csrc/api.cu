@@ -53,9 +53,10 @@ struct geo_mesh {
   double* adj_It = nullptr;  // stored Picard iterates of the node-team reverse sweep
   double ms[geo::N_STAGES] = {};
   int64_t cnt[geo::N_STAGES] = {};
-  // physical-state flag of the last step, copied to pinned host memory after
-  // each step and looked at by the next geo_step once that copy has landed
+  // physical-state flag of the last step, written to pinned host memory by each step's
+  // last kernel and looked at by the next geo_step once that kernel has finished
   int* status_host = nullptr;
+  double* scalar_host = nullptr;  // result of a device reduction (pinned)
   cudaEvent_t status_ev = nullptr;
   bool status_pending = false;
 
@@ -98,6 +99,8 @@ struct geo_mesh {
     allocs.clear();
     if (status_host) cudaFreeHost(status_host);
     status_host = nullptr;
+    if (scalar_host) cudaFreeHost(scalar_host);
+    scalar_host = nullptr;
     if (status_ev) cudaEventDestroy(status_ev);
     status_ev = nullptr;
     for (auto& t : pending) {
@@ -189,6 +192,8 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
     for (int c = 0; c < T.ncol; ++c) iV0[c] = 1.0 / T.V0[c];
     D.iq3 = m->upload(iq3, err);
     D.iV0 = m->upload(iV0, err);
+    for (int c = 0; c < T.ncol; ++c) iV0[c] = 6.0 * T.V0[c] / T.S0[c];
+    D.dz0 = m->upload(iV0, err);
     D.iA0 = m->upload(iA0, err);
     D.iq2 = m->upload(iq2, err);
   }
@@ -390,9 +395,15 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   S.Uhl = f32 ? static_cast<float*>(m->alloc_bytes(sizeof(float) * 16 * Z, err)) : nullptr;
   m->dt.status = static_cast<int*>(m->alloc_bytes(sizeof(int), err));
   if (err == cudaSuccess) err = cudaMemset(m->dt.status, 0, sizeof(int));
+  S.ticket = static_cast<unsigned*>(m->alloc_bytes(sizeof(unsigned), err));
+  if (err == cudaSuccess) err = cudaMemset(S.ticket, 0, sizeof(unsigned));
   if (err == cudaSuccess) err = cudaMallocHost(&m->status_host, sizeof(int));
+  if (err == cudaSuccess) err = cudaMallocHost(&m->scalar_host, sizeof(double));
   if (err == cudaSuccess) {
     *m->status_host = 0;
+    S.status_out = m->status_host;
+    S.host_out = m->scalar_host;
+    S.hl_fresh = true;
     err = cudaEventCreateWithFlags(&m->status_ev, cudaEventDisableTiming);
   }
   if (err != cudaSuccess) {
@@ -512,6 +523,7 @@ int geo_state_upload(geo_mesh_t m, const double* U, const double* phi, int on_de
   if (e != cudaSuccess) return cuda_fail(e, "state upload");
   m->status_pending = false;
   *m->status_host = 0;
+  m->ds.hl_fresh = true;
   m->have_state = true;
   return GEO_OK;
 }
@@ -547,9 +559,9 @@ int geo_step(geo_mesh_t m, double dt) {
     int rc = run_stage(m, s, dt);
     if (rc != GEO_OK) return rc;
   }
-  cudaError_t e = cudaMemcpyAsync(m->status_host, m->dt.status, sizeof(int), cudaMemcpyDeviceToHost, m->st);
-  if (e == cudaSuccess) e = cudaEventRecord(m->status_ev, m->st);
-  if (e != cudaSuccess) return cuda_fail(e, "status copy");
+  m->ds.hl_fresh = true;
+  cudaError_t e = cudaEventRecord(m->status_ev, m->st);
+  if (e != cudaSuccess) return cuda_fail(e, "status event");
   m->status_pending = true;
   return GEO_OK;
 }
@@ -832,6 +844,8 @@ int geo_debug_set_buffer(geo_mesh_t m, int which, const double* host, int64_t co
 int geo_debug_run_stage(geo_mesh_t m, int stage, double dt) {
   if (!m || stage < 0 || stage >= geo::N_STAGES) return fail(GEO_ERR_ARG, "bad arguments");
   cudaError_t e;
+  if (stage == geo::ST_ADER) m->ds.hl_fresh = false;
+  if (stage == geo::ST_UPD_U) m->ds.hl_fresh = true;
   switch (m->order) {
     case 2: e = m->prec == GEO_FP64 ? geo::launch_stage<2, double>(stage, m->dt, m->ds, dt, m->st)
                                     : geo::launch_stage<2, float>(stage, m->dt, m->ds, dt, m->st); break;

@@ -80,6 +80,7 @@ struct DevTables {
   const double* iq2;   // [nr + 2]: q^-2k
   const double* iq3;   // [nr + 2]: q^-3k
   const double* iV0;   // [ncol]: 1 / V0
+  const double* dz0;   // [ncol]: in-sphere diameter 6 V0 / S0 of the zone at shell 0
   const double *D, *R, *wt, *psiF, *psiE, *wE;
   const int* st_n;
   const int* st_nb;
@@ -110,6 +111,10 @@ struct DevState {
   double* Ff;    // [8][F] time-integrated face fluxes (FP64 accumulation)
   double* Ee;    // [E]   time-integrated edge EMFs (FP64 accumulation)
   double* red;   // reduction scratch
+  unsigned* ticket;   // [1] zero between reductions: blocks that have finished
+  double* host_out;   // [1] pinned host word that takes a reduction's result
+  int* status_out;    // [1] pinned host word that takes the physical-state flag after each step
+  bool hl_fresh;      // Uhl is the split of U (a predictor run alone changes U's field)
   float* Uhl;    // FP32-bulk only: [16][Z] U split as hi = fl(U), lo = fl(U - hi), for the WENO differences
 };
 
