@@ -1423,7 +1423,8 @@ __device__ __forceinline__ double warp_max(double v) {
 // FP32-bulk meshes first estimate each zone's time step in FP32 from the high parts of
 // the state's split; only zones within 1 % of the warp's smallest estimate so far (the
 // estimate is good to 0.1 %, the pressure's cancellation included) and those whose
-// estimate is not a positive number are evaluated in FP64, so the result is the same
+// estimate is not a positive number or has squares near FP32's underflow are evaluated
+// in FP64, so the result is the same
 // and the FP64 square roots and divisions run once or twice per warp instead of for
 // every zone (1,327,104 zones: 213 -> 89 us).
 __global__ void __launch_bounds__(RED_TPB) k_cfl(const DevTables T, const double* __restrict__ U,
@@ -1446,16 +1447,16 @@ __global__ void __launch_bounds__(RED_TPB) k_cfl(const DevTables T, const double
 #pragma unroll
       for (int v = 0; v < 8; ++v) h[v] = Uhl[v * Z + z];
       const float g = static_cast<float>(T.gamma), ir = 1.f / h[0];
-      const float m2 = (h[1] * h[1] + h[2] * h[2] + h[3] * h[3]) * ir;
+      const float vx = h[1] * ir, vy = h[2] * ir, vz = h[3] * ir;
       const float b2 = h[5] * h[5] + h[6] * h[6] + h[7] * h[7];
-      const float p = (g - 1.f) * (h[4] - 0.5f * m2 - 0.5f * b2);
-      const float e = static_cast<float>(T.dz0[c]) * static_cast<float>(T.qpow[k]) /
-                      (sqrtf(m2 * ir) + sqrtf((g * p + b2) * ir));
+      const float p = (g - 1.f) * ((h[4] - 0.5f * b2) - 0.5f * (h[1] * vx + h[2] * vy + h[3] * vz));
+      const float v2 = vx * vx + vy * vy + vz * vz, c2 = (g * p + b2) * ir;
+      const float e = static_cast<float>(T.dz0[c]) * static_cast<float>(T.qpow[k]) / (sqrtf(v2) + sqrtf(c2));
       float m = e > 0.f ? e : FLT_MAX;  // a NaN estimate does not hide the others
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
       near = fminf(near, m);
-      look = !(e > 1.01f * near);
+      look = !(e > 1.01f * near) || !(v2 + c2 > 1e-30f);
     }
     if (look) {
       double u[8];
