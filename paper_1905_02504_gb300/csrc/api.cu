@@ -136,6 +136,19 @@ static int run_stage(geo_mesh* m, int stage, double dt) {
   return GEO_OK;
 }
 
+// faces, edges and updates of a small mesh in two launches; false where it is not small
+static bool corrector_small(geo_mesh* m, double dt, cudaError_t& e) {
+  const bool f32 = m->prec == GEO_FP32_BULK;
+  switch (m->order) {
+    case 2: return f32 ? geo::launch_corrector_small<2, float>(m->dt, m->ds, dt, m->st, e)
+                       : geo::launch_corrector_small<2, double>(m->dt, m->ds, dt, m->st, e);
+    case 3: return f32 ? geo::launch_corrector_small<3, float>(m->dt, m->ds, dt, m->st, e)
+                       : geo::launch_corrector_small<3, double>(m->dt, m->ds, dt, m->st, e);
+    default: return f32 ? geo::launch_corrector_small<4, float>(m->dt, m->ds, dt, m->st, e)
+                        : geo::launch_corrector_small<4, double>(m->dt, m->ds, dt, m->st, e);
+  }
+}
+
 namespace geo {
 // accessors used by the allocation-free entry point (noalloc.cu)
 const DevTables* mesh_dev_tables(const geo_mesh* m) { return &m->dt; }
@@ -556,6 +569,13 @@ int geo_step(geo_mesh_t m, double dt) {
     if (*m->status_host) return fail(GEO_ERR_NONPHYSICAL, "an earlier step produced a non-physical state");
   }
   for (int s = 0; s < geo::N_STAGES; ++s) {
+    if (s == geo::ST_FACE && !m->timing) {  // stage timing needs a launch per stage
+      cudaError_t ce = cudaSuccess;
+      if (corrector_small(m, dt, ce)) {
+        if (ce != cudaSuccess) return cuda_fail(ce, "kernel launch");
+        break;
+      }
+    }
     int rc = run_stage(m, s, dt);
     if (rc != GEO_OK) return rc;
   }

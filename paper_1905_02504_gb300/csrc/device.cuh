@@ -147,6 +147,10 @@ cudaError_t upload_reference_constants(const Tables& T);
 // launchers (kernels.cu); return cudaGetLastError() of the launch
 template <int P, typename R>
 cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, double dt, cudaStream_t st);
+// stages ST_FACE .. ST_UPD_PHI of a small mesh in two launches; false (nothing launched)
+// where the mesh is not small
+template <int P, typename R>
+bool launch_corrector_small(const DevTables& T, const DevState& S, double dt, cudaStream_t st, cudaError_t& e);
 // the FP64 predictor (no positivity) that also stores its Picard
 // iterates for the reverse sweep (It: [P-1][M-1][8][N][Z] doubles)
 template <int P>
