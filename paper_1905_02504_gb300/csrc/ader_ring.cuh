@@ -33,7 +33,7 @@
 //   FP32 p = 4, 147,456 zones  2446 -> 1288 us     FP64 p = 4, 110,592 zones  26.98 -> 20.95 ms
 //   FP32 p = 3, 193,536 zones   705 ->  581 us     FP64 p = 3, 193,536 zones  13.23 -> 10.99 ms
 //   FP32 p = 2, 1,327,104 zones 1023 -> 917 us     FP64 p = 2, 165,888 zones   1.75 ->  1.78 ms
-// With positivity: FP32 p = 4 (55,296 zones) 1031 -> 779 us, FP64 p = 4 (18,432)
+// With positivity: FP32 p = 4 (55,296 zones) 1031 -> 688 us, FP64 p = 4 (18,432)
 // 4.99 -> 3.99 ms, FP64 p = 3 (73,728) 5.90 -> 5.35 ms; at FP32 p = 3 and at p = 2 the
 // node team stays ahead (419 against 427 us, 166 against 209 us).
 
@@ -232,9 +232,9 @@ __device__ __forceinline__ void ring_contract(R* Fz, int lane) {
 // and to face q's edge (and, shared out, the middle one).  A warp has one q and, as
 // lanes, four zones x 8 variables: by the symmetry of the element all q use the same
 // weights (constant bank), the point's index is uniform, and a store fills whole
-// 128-byte lines of [point][zone][8].  face / edge(idx, m0, s): the point's values at
-// the levels m0...
-template <int P, int ML, typename R, typename EmitF, typename EmitE>
+// 128-byte lines of [point][zone][8].  face / edge(idx, m0, s, mine): the point's values
+// at the levels m0..; with ALL every q passes every point, mine telling whose it is.
+template <int P, int ML, bool ALL, typename R, typename EmitF, typename EmitE>
 __device__ __forceinline__ void ring_points(const R* Fz, int q, const RefConst<P, R>& K, EmitF&& face,
                                             EmitE&& edge) {
   using L = RingLayout<P, R>;
@@ -268,7 +268,7 @@ __device__ __forceinline__ void ring_points(const R* Fz, int q, const RefConst<P
 #pragma unroll
           for (int t = 0; t < G::PS; ++t) s[m] += w[2 * P + t] * p0[m][t];
         }
-        face(base + a * du + b, 0, s);
+        face(base + a * du + b, 0, s, true);
       }
     // ---- edges: radial edge q, then bottom and top edge of face q
 #pragma unroll
@@ -295,7 +295,7 @@ __device__ __forceinline__ void ring_points(const R* Fz, int q, const RefConst<P
             for (int t = 1; t < P; ++t) val[m] += K.wEd[s * P + t] * y[t];
           }
         }
-        edge(b0 + s * ds, 0, val);
+        edge(b0 + s * ds, 0, val, true);
       }
     }
   }
@@ -309,7 +309,7 @@ __device__ __forceinline__ void ring_points(const R* Fz, int q, const RefConst<P
 #pragma unroll
     for (int top = 0; top < 2; ++top) {
       const int f0 = 4 * Dm::NQS + top * Dm::NQR;
-      auto point = [&](int w3, int idx) {
+      auto point = [&](int w3, int idx, bool mine) {
         const R* w = K.wR + w3 * NFN;
         R s[1] = {R(0)};
 #pragma unroll
@@ -318,16 +318,41 @@ __device__ __forceinline__ void ring_points(const R* Fz, int q, const RefConst<P
 #pragma unroll
           for (int t = 0; t < PI; ++t) s[0] += w[4 + r * PI + t] * p[r][top * PI + t];
         }
-        face(f0 + idx, m, s);
+        face(f0 + idx, m, s, mine);
       };
-      point(0, G::bit_b(q) * (NU - 1) * NU + G::bit_c(q) * (NU - 1));
+      point(0, G::bit_b(q) * (NU - 1) * NU + G::bit_c(q) * (NU - 1), true);
       if constexpr (P == 4) {
         // next to the middle of face q's edge: (1,0), (2,1), (1,2), (0,1)
-        point(1, (q == 1 ? 2 : (q == 3 ? 0 : 1)) * NU + (q == 0 ? 0 : (q == 2 ? 2 : 1)));
-        if (q == 2 * top) point(2, NU + 1);
+        point(1, (q == 1 ? 2 : (q == 3 ? 0 : 1)) * NU + (q == 0 ? 0 : (q == 2 ? 2 : 1)), true);
+        if (ALL || q == 2 * top) point(2, NU + 1, q == 2 * top);
       }
     }
   }
+}
+
+// Positivity factors of the point states held in a warp's tile (lane = zone * 8 + slot),
+// min-reduced into the zones' th: pass 0 theta_rho and, for theta_rho = 1, theta_p;
+// pass 1 theta_p for the zone's theta_rho.  Out of line: it is called every SLOTS points
+// of the fully unrolled point code, which it would blow up beyond the instruction cache.
+template <int P, typename R>
+__device__ __noinline__ void ring_check(const R* my, RingSmem<P, R>& S, int held, int zl, int lane, R gam, int pass) {
+  constexpr int TS = RingTile<P, R, true>::STRIDE;
+  __syncwarp();
+  if ((lane & 7) < held) {
+    R s[8], mz[8];
+    ld8(my + (lane & 7) * TS + (lane & 24), s);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) mz[e] = S.Uz[e][zl];
+    const R pb = pressure_of(mz, gam), er = fmin(R(1e-13), mz[0]), ep = fmin(R(1e-13), pb);
+    R pr = R(1), pp = R(1);
+    if (pass == 0) {
+      pos_rho(s, mz, er, pr);
+      if (pr < R(1)) smem_min_nonneg(&S.th[zl][2], pr);
+    }
+    pos_p(s, mz, pass == 0 ? R(1) : S.th[zl][2], gam, pb, ep, pp);
+    if (pp < R(1)) smem_min_nonneg(&S.th[zl][pass == 0 ? 4 : 3], pp);
+  }
+  __syncwarp();
 }
 
 // STORE: also write the levels (times J) after each of the first P-1 Picard iterations to
@@ -766,26 +791,21 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
     const bool in = zbase + zt < Z;
     if (!in) ct = c0;
     const size_t at = static_cast<size_t>(zbase + (t >> 2) * 4) * 8 + (P == 4 ? lane : 0);
-    const int mine = P == 4 ? 0 : lane;  // the task's 4 x 8 values, one per lane
+    const int off = P == 4 ? 0 : lane;  // the task's 4 x 8 values, one per lane
     const R* iJF = BT.iJF + static_cast<size_t>(ct) * NQT;
     const R* iJE = BT.iJE + static_cast<size_t>(ct) * 12 * Dm::NS;
     // (1/J through the read-only path: the compiler may then keep it across the stores)
-    auto put = [&](const R* iJ, R* out, size_t step, int idx, int m0, const auto& s) {
+    auto put = [&](const R* iJ, R* out, size_t step, int idx, int m0, const auto& s, bool mine) {
       const R w = __ldg(iJ + idx);
       R* o = out + at + static_cast<size_t>(static_cast<unsigned>(idx)) * Z8;
 #pragma unroll
-      for (int m = 0; m < static_cast<int>(sizeof(s) / sizeof(R)); ++m) emit(in, s[m] * w, o + (m0 + m) * step + mine);
+      for (int m = 0; m < static_cast<int>(sizeof(s) / sizeof(R)); ++m) emit(in && mine, s[m] * w, o + (m0 + m) * step + off);
     };
     const R* row = S.F + zt * L::FL + v * L::RS;
-    // all levels together share the weights' and addresses' work; with positivity, whose
-    // checks are inlined at every point, one level at a time keeps the code within the
-    // instruction cache (p = 4 FP32, low-beta blast, 55,296 zones: 1047 -> 779 us)
-    constexpr int NL = POS ? 1 : ML;
-#pragma unroll 1
-    for (int l = 0; l < ML; l += NL)
-      ring_points<P, NL>(
-          row + l * L::FS, q, K, [&](int idx, int m0, const auto& s) { put(iJF, trF, ZF, idx, l + m0, s); },
-          [&](int idx, int m0, const auto& s) { put(iJE, trE, ZE, idx, l + m0, s); });
+    ring_points<P, ML, POS>(
+        row, q, K,
+        [&](int idx, int m0, const auto& s, bool mine) { put(iJF, trF, ZF, idx, m0, s, mine); },
+        [&](int idx, int m0, const auto& s, bool mine) { put(iJE, trE, ZE, idx, m0, s, mine); });
   };
   static_assert(ZB % 4 == 0, "zones in fours");
   if constexpr (!POS) {
@@ -813,42 +833,26 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
 #pragma unroll 1
       for (int t = warp; t < ZB; t += NW) {
         const int zt = (t >> 2) * 4 + (lane >> 3);
-        R mz[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) mz[e] = S.Uz[e][zt];
-        const R um = S.Uz[v][zt], pb = pressure_of(mz, gam);
-        const R er = fmin(R(1e-13), mz[0]), ep = fmin(R(1e-13), pb);
-        const R th_r = pass == 0 ? R(1) : S.th[zt][2];
+        const R um = S.Uz[v][zt], th_r = S.th[zt][2];
         const R th = pass < 2 ? R(1) : th_r * (th_r < R(1) ? S.th[zt][3] : S.th[zt][4]);
-        R pr = R(1), pp = R(1);
         R* my = tile.s[warp];
-        constexpr int TS = RingTile<P, R, POS>::STRIDE;
-        int held = 0;  // point states of each zone in the tile
-        auto check = [&]() {
-          __syncwarp();
-          if (v < held) {
-            R s[8];
-            ld8(my + v * TS + (lane & 24), s);
-            if (pass == 0) pos_rho(s, mz, er, pr);
-            pos_p(s, mz, th_r, gam, pb, ep, pp);
-          }
-          held = 0;
-          __syncwarp();
-        };
-        task(t, [&](bool in, R x, R* out) {
-          if (pass < 2) {
-            my[held * TS + lane] = x;
-            if (++held == RingTile<P, R, POS>::SLOTS) check();
-          }
-          if (in && pass == 0) *out = x;
-          if (in && pass == 2 && th < R(1)) *out = um + th * (x - um);
-        });
+        constexpr int TS = RingTile<P, R, POS>::STRIDE, SLOTS = RingTile<P, R, POS>::SLOTS;
+        const bool inside = zbase + zt < Z;  // a whole octet of lanes
         if (pass < 2) {
-          check();
-          if (zbase + zt < Z) {
-            if (pass == 0 && pr < R(1)) smem_min_nonneg(&S.th[zt][2], pr);
-            if (pp < R(1)) smem_min_nonneg(&S.th[zt][pass == 0 ? 4 : 3], pp);
-          }
+          int held = 0;  // point states of each zone in the tile
+          task(t, [&](bool in, R x, R* out) {
+            my[held * TS + lane] = x;
+            if (++held == SLOTS) {
+              ring_check<P, R>(my, S, inside ? held : 0, zt, lane, gam, pass);
+              held = 0;
+            }
+            if (in && pass == 0) *out = x;
+          });
+          ring_check<P, R>(my, S, inside ? held : 0, zt, lane, gam, pass);
+        } else {
+          task(t, [&](bool in, R x, R* out) {
+            if (in && th < R(1)) *out = um + th * (x - um);
+          });
         }
       }
       __syncthreads();
