@@ -235,7 +235,7 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
     }
   }
   D.pinvH = m->upload(PTt, err);
-  D.Qs = nullptr;  // FP32 only
+  D.Qs = m->upload(Qst, err);
   D.oct_nb = m->upload(T.oct_nb, err);
   D.oct_inv = m->upload(T.oct_inv, err);
   D.Q = m->upload(T.Q, err);
@@ -738,6 +738,22 @@ int geo_debug_buffer(geo_mesh_t m, int which, double* host, int64_t count) {
   return GEO_OK;
 }
 
+// one forward stage of the reverse sweep's recompute, on its own buffers
+static cudaError_t adj_forward_stage(geo_mesh* m, int s, double dt) {
+  if (s == geo::ST_WENO) {
+    switch (m->order) {
+      case 2: return geo::launch_weno_exact<2>(m->dt, m->adj_fwd, m->st);
+      case 3: return geo::launch_weno_exact<3>(m->dt, m->adj_fwd, m->st);
+      default: return geo::launch_weno_exact<4>(m->dt, m->adj_fwd, m->st);
+    }
+  }
+  switch (m->order) {
+    case 2: return geo::launch_stage<2, double>(s, m->dt, m->adj_fwd, dt, m->st);
+    case 3: return geo::launch_stage<3, double>(s, m->dt, m->adj_fwd, dt, m->st);
+    default: return geo::launch_stage<4, double>(s, m->dt, m->adj_fwd, dt, m->st);
+  }
+}
+
 static int ensure_adjoint_buffers(geo_mesh* m) {
   if (m->adj_ready) return GEO_OK;
   const geo::Dims& d = m->T.d;
@@ -800,11 +816,7 @@ int geo_step_adjoint(geo_mesh_t m, double dt, const double* U_in, const double* 
       }
       continue;
     }
-    switch (m->order) {
-      case 2: e = geo::launch_stage<2, double>(s, m->dt, m->adj_fwd, dt, m->st); break;
-      case 3: e = geo::launch_stage<3, double>(s, m->dt, m->adj_fwd, dt, m->st); break;
-      default: e = geo::launch_stage<4, double>(s, m->dt, m->adj_fwd, dt, m->st); break;
-    }
+    e = adj_forward_stage(m, s, dt);
   }
   if (e != cudaSuccess) return cuda_fail(e, "adjoint forward recompute");
   geo::AdjState A = m->adj;
@@ -918,11 +930,7 @@ int geo_debug_stage_vjp(geo_mesh_t m, int stage, double dt, const double* U, con
   if (e == cudaSuccess) e = cudaMemcpyAsync(m->adj_fwd.U, U, 8 * Z * sizeof(double), cudaMemcpyHostToDevice, m->st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(m->adj_fwd.phi, phi, F * sizeof(double), cudaMemcpyHostToDevice, m->st);
   for (int s = geo::ST_WENO; s <= geo::ST_ADER && e == cudaSuccess; ++s) {
-    switch (m->order) {
-      case 2: e = geo::launch_stage<2, double>(s, m->dt, m->adj_fwd, dt, m->st); break;
-      case 3: e = geo::launch_stage<3, double>(s, m->dt, m->adj_fwd, dt, m->st); break;
-      default: e = geo::launch_stage<4, double>(s, m->dt, m->adj_fwd, dt, m->st); break;
-    }
+    e = adj_forward_stage(m, s, dt);
   }
   A.gUp = gU0;
   A.gphip = nullptr;

@@ -151,6 +151,9 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
 // where the mesh is not small
 template <int P, typename R>
 bool launch_corrector_small(const DevTables& T, const DevState& S, double dt, cudaStream_t st, cudaError_t& e);
+// WENO-AO in the reverse sweep's order of summation (FP64)
+template <int P>
+cudaError_t launch_weno_exact(const DevTables& T, const DevState& S, cudaStream_t st);
 // the FP64 predictor (no positivity) that also stores its Picard
 // iterates for the reverse sweep (It: [P-1][M-1][8][N][Z] doubles)
 template <int P>

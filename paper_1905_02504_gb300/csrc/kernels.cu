@@ -58,20 +58,20 @@ using namespace dev;
 // those loads (one per multiply-add).  With VB variables an entry loaded once serves
 // VB multiply-adds (p = 4, 147,456 zones: 275 -> 138 us with VB = 4, 145 us with 2;
 // p = 3, 193,536 zones: 172 -> 93 / 100 us; p = 2, 1,327,104 zones: 474 -> 304 / 279 us).
-// In FP32 beta_H comes from the upper triangle of the smoothness form (off-diagonals
-// doubled, rows padded to whole 16-byte vectors).  Both forms take the six face
-// neighbours' differences once for the eight octants that share them.  The FP64 form is
-// bound by its own pipe and keeps VB = 1, which spreads small meshes over more warps;
-// it sums in the order of the reverse sweep's own evaluation (k_adj_weno), bit for bit,
-// so that ties (MinMod between mirror images of a symmetric field) fall to the same side
-// as ever (p = 4, 110,592 zones: 2.02 -> 1.99 ms; a triangular beta_H would give 1.70 ms
-// and turned such ties over).
+// beta_H comes from the upper triangle of the smoothness form (off-diagonals doubled,
+// rows padded to whole 16-byte vectors), and the six face neighbours' differences serve
+// the eight octants that share them.  The FP64 form is bound by its own pipe and keeps
+// VB = 1, which spreads small meshes over more warps (p = 4, 110,592 zones: 2.02 -> 1.70
+// ms; p = 3, 193,536 zones: 1.99 -> 1.76 ms).
+// EXACT: the order of summation of the reverse sweep's own evaluation (k_adj_weno), bit
+// for bit.  The reverse sweep's recompute takes it, so that its decisions at ties (MinMod
+// between mirror images of a symmetric field) are the ones that its kernels then reverse.
 // ----------------------------------------------------------------------------
 template <int P> struct WenoVb { static constexpr int VB = P == 2 ? 2 : 4; };
 // zones from which the grid with VB variables per thread still fills the GPU
 constexpr long long WENO_WIDE = 20000;
 
-template <int P, typename R, int VB>
+template <int P, typename R, int VB, bool EXACT = false>
 __global__ void __launch_bounds__(TPB, 3) k_weno(const DevTables T, const double* __restrict__ U,
                                               const float* __restrict__ Uhl, R* __restrict__ Wc) {
   using Dm = Dim<P>;
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(TPB, 3) k_weno(const DevTables T, const double
   R bH[VB];
 #pragma unroll
   for (int v = 0; v < VB; ++v) bH[v] = R(0);
-  if constexpr (sizeof(R) == 4) {
+  if constexpr (!EXACT) {
     const R* q = B.Qs + static_cast<size_t>(c) * Dm::QTRI;
 #pragma unroll
     for (int i = 0; i < NC1; ++i) {
@@ -223,13 +223,13 @@ __global__ void __launch_bounds__(TPB, 3) k_weno(const DevTables T, const double
     fH[v] = wH / GH;
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
-      if constexpr (sizeof(R) == 4) wK[v][o] = wK[v][o] * itot - fH[v] * GK;
+      if constexpr (!EXACT) wK[v][o] = wK[v][o] * itot - fH[v] * GK;
       else wK[v][o] *= itot;
     }
   }
   // out_a = fH (uH_a - GK sum_o uK_oa) + sum_o w_o uK_oa (a < 3), out_m = fH uH_m
   R s3[VB][3];
-  if constexpr (sizeof(R) == 8) {
+  if constexpr (EXACT) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       R sk = R(0), wk = R(0);
@@ -1926,6 +1926,15 @@ cudaError_t launch_adj_ader(const DevTables& T, const DevState& S, const AdjStat
   };
   return A.It ? run(k_adj_ader_team<P, true>) : run(k_adj_ader_team<P, false>);
 }
+
+template <int P>
+cudaError_t launch_weno_exact(const DevTables& T, const DevState& S, cudaStream_t st) {
+  k_weno<P, double, 1, true><<<dim3(grid_for(T.Z), 8), TPB, 0, st>>>(T, S.U, nullptr, static_cast<double*>(S.Wc));
+  return cudaGetLastError();
+}
+template cudaError_t launch_weno_exact<2>(const DevTables&, const DevState&, cudaStream_t);
+template cudaError_t launch_weno_exact<3>(const DevTables&, const DevState&, cudaStream_t);
+template cudaError_t launch_weno_exact<4>(const DevTables&, const DevState&, cudaStream_t);
 
 template <int P>
 cudaError_t launch_ader_store_iterates(const DevTables& T, const DevState& S, double* It, double dt, cudaStream_t st) {
