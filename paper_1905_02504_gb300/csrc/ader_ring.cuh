@@ -31,8 +31,8 @@
 // Measured, predictor alone, against the sparse rows on the compiled pattern of D^alpha
 // (FP64 p = 4: the node team's padded rows):
 //   FP32 p = 4, 147,456 zones  2446 -> 1288 us     FP64 p = 4, 110,592 zones  26.98 -> 20.95 ms
-//   FP32 p = 3, 193,536 zones   705 ->  581 us     FP64 p = 3, 193,536 zones  13.23 -> 10.99 ms
-//   FP32 p = 2, 1,327,104 zones 1023 -> 917 us     FP64 p = 2, 165,888 zones   1.75 ->  1.78 ms
+//   FP32 p = 3, 193,536 zones   705 ->  561 us     FP64 p = 3, 193,536 zones  13.23 -> 10.99 ms
+//   FP32 p = 2, 1,327,104 zones 1023 -> 822 us     FP64 p = 2, 165,888 zones   1.75 ->  1.78 ms
 // With positivity: FP32 p = 4 (55,296 zones) 1031 -> 688 us, FP64 p = 4 (18,432)
 // 4.99 -> 3.99 ms, FP64 p = 3 (73,728) 5.90 -> 5.35 ms; at FP32 p = 3 and at p = 2 the
 // node team stays ahead (419 against 427 us, 166 against 209 us).
@@ -83,7 +83,7 @@ struct Ring {
 // lane = node.  P = 3: a warp holds four nodes of the block's eight zones (zone
 // fastest); P = 2: eight nodes of four zones.
 template <int P, typename R> struct RingCfg;
-template <> struct RingCfg<2, float> { static constexpr bool POS = false, WARP = false; static constexpr int ZB = 16, MINB = 12; };
+template <> struct RingCfg<2, float> { static constexpr bool POS = false, WARP = false; static constexpr int ZB = 16, MINB = 14; };
 template <> struct RingCfg<3, float> { static constexpr bool POS = false, WARP = false; static constexpr int ZB = 8, MINB = 7; };
 template <> struct RingCfg<4, float> { static constexpr bool POS = true, WARP = true; static constexpr int ZB = 4, MINB = 5; };
 template <> struct RingCfg<2, double> { static constexpr bool POS = false, WARP = false; static constexpr int ZB = 16, MINB = 4; };
