@@ -280,19 +280,12 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   D.se_le = m->upload(T.se_le, err);
   D.se_rev = m->upload(T.se_rev, err);
   D.se_t = m->upload(T.se_t, err);
-  D.se_dlw = m->upload(T.se_dlw, err);
   D.se_nang = m->upload(T.se_nang, err);
   D.se_nradL = m->upload(T.se_nradL, err);
   D.se_nradR = m->upload(T.se_nradR, err);
   D.sv_nc = m->upload(T.sv_nc, err);
-  D.sv_col = m->upload(T.sv_col, err);
-  D.sv_le = m->upload(T.sv_le, err);
-  D.sv_fL = m->upload(T.sv_fL, err);
-  D.sv_fR = m->upload(T.sv_fR, err);
   D.sv_fse = m->upload(T.sv_fse, err);
-  D.sv_fn = m->upload(T.sv_fn, err);
   D.sv_t = m->upload(T.sv_t, err);
-  D.sv_dlw = m->upload(T.sv_dlw, err);
   // radial edges in ring order, with each face's normal turned to point from its first
   // to its second ring zone
   const int NS = d.NS, M1 = d.M - 1;

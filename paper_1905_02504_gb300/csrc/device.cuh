@@ -89,9 +89,9 @@ struct DevTables {
   const double *oct_inv, *Q, *Qs, *V0, *l0, *S0, *A0, *TF, *nF, *wF, *WF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
   const int *col_side_se, *col_side_sgn;
   const int *se_v, *se_col, *se_lf, *se_perm, *se_le, *se_rev;
-  const double *se_t, *se_dlw, *se_nang, *se_nradL, *se_nradR;
-  const int *sv_nc, *sv_col, *sv_le, *sv_fL, *sv_fR, *sv_fse;
-  const double *sv_fn, *sv_t, *sv_dlw;
+  const double *se_t, *se_nang, *se_nradL, *se_nradR;
+  const int *sv_nc, *sv_fse;
+  const double* sv_t;
   // zones around a radial edge in ring order (face j between zones j and j + 1; three
   // zones: the fourth entry repeats the first): column, local edge [nsv][4]
   const int *svr_col, *svr_le;

@@ -1188,16 +1188,10 @@ __global__ void __launch_bounds__(TPB) k_face_flux(const DevTables T, const R* _
 // ----------------------------------------------------------------------------
 constexpr long long EDGE_SPLIT_MAX = 40000;
 
-template <int P, typename R, int SPLIT>
-__device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict__ trE, double* __restrict__ Ee,
-                                         double dt, long long t0) {
-  using Dm = Dim<P>;
-  constexpr int M = Dm::M, NS = Dm::NS, NP = (M - 1) * NS;
-  const long long E = T.E, Z = T.Z;
-  const long long e = t0 / SPLIT < E ? t0 / SPLIT : E - 1;
-  const int nr = T.nr;
-  const R g = static_cast<R>(T.gamma);
-  const BulkTables<R>& BT = bulk<R>(T);
+// the zones and faces around edge e in ring order
+template <int P, typename R>
+struct EdgeRing {
+  static constexpr int NS = Dim<P>::NS, NP = (Dim<P>::M - 1) * NS;
   long long zs[4];
   int le[4];          // first edge point of the zone's local edge, or the last one if reversed
   int rev = 0;        // bit j: zone j counts the points from the other end
@@ -1206,68 +1200,89 @@ __device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict
   R fs[4] = {R(1), R(1), R(1), R(1)};  // their sign
   const R *tv, *tw;   // tangents (one for a radial edge), weights [M-1][NS]
   int ts;             // stride of the tangents
-  double q;
-  if (e < T.E_rad) {
-    int sv, k;
-    zone_column(e, nr, sv, k);
-    nz = T.sv_nc[sv];
-    nf = nz;
+  double q;           // radial scale of the weights
+
+  __device__ __forceinline__ EdgeRing(const DevTables& T, long long e) {
+    const int nr = T.nr;
+    const BulkTables<R>& BT = bulk<R>(T);
+    if (e < T.E_rad) {
+      int sv, k;
+      zone_column(e, nr, sv, k);
+      nz = T.sv_nc[sv];
+      nf = nz;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      zs[j] = static_cast<long long>(T.svr_col[4 * sv + j]) * nr + k;
-      le[j] = T.svr_le[4 * sv + j] * NS;
-      fn[j] = BT.svr_fn + static_cast<size_t>(sv * 4 + j) * NS * 3;
-    }
-    tv = BT.sv_t + 3 * sv;
-    ts = 0;
-    tw = BT.sv_w + static_cast<size_t>(sv) * NP;
-    q = T.qpow[k];
-  } else {
-    int se, kk;
-    zone_column(e - T.E_rad, nr + 1, se, kk);
-    const int cL = T.se_col[2 * se], cR = T.se_col[2 * se + 1];
-    const int rL = T.se_rev[2 * se], rR = T.se_rev[2 * se + 1];
-    const R* nang = BT.se_nang + static_cast<size_t>(se) * NS * 3;
-    if (kk >= 1 && kk <= nr - 1) {
-      // ring: L below, L above, R above, R below
-      nz = nf = 4;
-      zs[0] = static_cast<long long>(cL) * nr + kk - 1; le[0] = T.se_le[4 * se + 1];
-      zs[1] = zs[0] + 1;                                le[1] = T.se_le[4 * se];
-      zs[3] = static_cast<long long>(cR) * nr + kk - 1; le[3] = T.se_le[4 * se + 3];
-      zs[2] = zs[3] + 1;                                le[2] = T.se_le[4 * se + 2];
-      rev = (rL ? 3 : 0) | (rR ? 12 : 0);
-      fn[0] = BT.se_nradL + static_cast<size_t>(se) * NS * 3;
-      fn[1] = fn[3] = nang;
-      fn[2] = BT.se_nradR + static_cast<size_t>(se) * NS * 3;
-      fs[2] = fs[3] = R(-1);
+      for (int j = 0; j < 4; ++j) {
+        zs[j] = static_cast<long long>(T.svr_col[4 * sv + j]) * nr + k;
+        le[j] = T.svr_le[4 * sv + j] * NS;
+        fn[j] = BT.svr_fn + static_cast<size_t>(sv * 4 + j) * NS * 3;
+      }
+      tv = BT.sv_t + 3 * sv;
+      ts = 0;
+      tw = BT.sv_w + static_cast<size_t>(sv) * NP;
+      q = T.qpow[k];
     } else {
-      nz = 2;
-      nf = 1;
-      const int top = kk == nr ? 1 : 0, kz = top ? nr - 1 : 0;
-      zs[0] = static_cast<long long>(cL) * nr + kz; le[0] = T.se_le[4 * se + top];
-      zs[1] = static_cast<long long>(cR) * nr + kz; le[1] = T.se_le[4 * se + 2 + top];
-      zs[2] = zs[3] = zs[0];
-      le[2] = le[3] = le[0];
-      rev = (rL ? 1 : 0) | (rR ? 2 : 0);
+      int se, kk;
+      zone_column(e - T.E_rad, nr + 1, se, kk);
+      const int cL = T.se_col[2 * se], cR = T.se_col[2 * se + 1];
+      const int rL = T.se_rev[2 * se], rR = T.se_rev[2 * se + 1];
+      const R* nang = BT.se_nang + static_cast<size_t>(se) * NS * 3;
+      if (kk >= 1 && kk <= nr - 1) {
+        // ring: L below, L above, R above, R below
+        nz = nf = 4;
+        zs[0] = static_cast<long long>(cL) * nr + kk - 1; le[0] = T.se_le[4 * se + 1];
+        zs[1] = zs[0] + 1;                                le[1] = T.se_le[4 * se];
+        zs[3] = static_cast<long long>(cR) * nr + kk - 1; le[3] = T.se_le[4 * se + 3];
+        zs[2] = zs[3] + 1;                                le[2] = T.se_le[4 * se + 2];
+        rev = (rL ? 3 : 0) | (rR ? 12 : 0);
+        fn[0] = BT.se_nradL + static_cast<size_t>(se) * NS * 3;
+        fn[1] = fn[3] = nang;
+        fn[2] = BT.se_nradR + static_cast<size_t>(se) * NS * 3;
+        fs[2] = fs[3] = R(-1);
+      } else {
+        nz = 2;
+        nf = 1;
+        const int top = kk == nr ? 1 : 0, kz = top ? nr - 1 : 0;
+        zs[0] = static_cast<long long>(cL) * nr + kz; le[0] = T.se_le[4 * se + top];
+        zs[1] = static_cast<long long>(cR) * nr + kz; le[1] = T.se_le[4 * se + 2 + top];
+        zs[2] = zs[3] = zs[0];
+        le[2] = le[3] = le[0];
+        rev = (rL ? 1 : 0) | (rR ? 2 : 0);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) fn[j] = nang;
+        for (int j = 0; j < 4; ++j) fn[j] = nang;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) le[j] *= NS;
+      tv = BT.se_t + static_cast<size_t>(se) * NS * 3;
+      ts = 3;
+      tw = BT.se_w + static_cast<size_t>(se) * NP;
+      q = T.qpow[kk];
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) le[j] *= NS;
-    tv = BT.se_t + static_cast<size_t>(se) * NS * 3;
-    ts = 3;
-    tw = BT.se_w + static_cast<size_t>(se) * NP;
-    q = T.qpow[kk];
+    for (int j = 0; j < 4; ++j)
+      if ((rev >> j) & 1) le[j] += NS - 1;
   }
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if ((rev >> j) & 1) le[j] += NS - 1;
+  // offset of zone j's state at point s of Gauss level m
+  __device__ __forceinline__ size_t at(int j, int m, int s, long long Z) const {
+    return trE_at<P>(zs[j], m, le[j] + (((rev >> j) & 1) ? -s : s), Z);
+  }
+};
+
+template <int P, typename R, int SPLIT>
+__device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict__ trE, double* __restrict__ Ee,
+                                         double dt, long long t0) {
+  using Dm = Dim<P>;
+  constexpr int NS = Dm::NS, NP = (Dm::M - 1) * NS;
+  const long long E = T.E, Z = T.Z;
+  const long long e = t0 / SPLIT < E ? t0 / SPLIT : E - 1;
+  const R g = static_cast<R>(T.gamma);
+  const EdgeRing<P, R> G(T, e);
+  const int nz = G.nz, nf = G.nf;
   const R inz = R(1) / static_cast<R>(nz);
   R acc = R(0);  // quadrature sum in the bulk type; the Phi update is FP64
 #pragma unroll 1
   for (int pt = SPLIT == 1 ? 0 : static_cast<int>(t0 % SPLIT); pt < NP; pt += SPLIT) {
     const int m = pt / NS + 1, s = pt % NS;
-    const R tx = tv[ts * s], ty = tv[ts * s + 1], tz = tv[ts * s + 2];
+    const R tx = G.tv[G.ts * s], ty = G.tv[G.ts * s + 1], tz = G.tv[G.ts * s + 2];
     // per zone: v, B, s = a^2 + b^2 and 4 a^2 / rho of the fast speed (1/rho formed once)
     R vx[4], vy[4], vz[4], bx[4], by[4], bz[4], sq[4], qa[4];
     R Ev = R(0);
@@ -1280,7 +1295,7 @@ __device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict
         continue;
       }
       R u[8];
-      ld8(trE + trE_at<P>(zs[j], m, le[j] + (((rev >> j) & 1) ? -s : s), Z), u);
+      ld8(trE + G.at(j, m, s, Z), u);
       const R ir = R(1) / u[0];
       vx[j] = u[1] * ir; vy[j] = u[2] * ir; vz[j] = u[3] * ir;
       bx[j] = u[5]; by[j] = u[6]; bz[j] = u[7];
@@ -1302,17 +1317,17 @@ __device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict
     for (int j = 0; j < 4; ++j) {
       if (j >= nf) continue;
       const int r = (j + 1) & 3;
-      const R* nv = fn[j] + 3 * s;
+      const R* nv = G.fn[j] + 3 * s;
       const R nx = nv[0], ny = nv[1], nzz = nv[2];
-      const R a = fs[j] * fmax(speed(j, nx, ny, nzz), speed(r, nx, ny, nzz));
+      const R a = G.fs[j] * fmax(speed(j, nx, ny, nzz), speed(r, nx, ny, nzz));
       // a (B_r - B_j) . (t x n)
       Ev += a * ((bx[r] - bx[j]) * (ty * nzz - tz * ny) + (by[r] - by[j]) * (tz * nx - tx * nzz) +
                  (bz[r] - bz[j]) * (tx * ny - ty * nx));
     }
-    acc += tw[pt] * (Ev * inz);
+    acc += G.tw[pt] * (Ev * inz);
   }
   acc = lane_sum<SPLIT>(acc);
-  if (t0 < E * SPLIT && (SPLIT == 1 || t0 % SPLIT == 0)) Ee[e] = dt * q * static_cast<double>(acc);
+  if (t0 < E * SPLIT && (SPLIT == 1 || t0 % SPLIT == 0)) Ee[e] = dt * G.q * static_cast<double>(acc);
 }
 
 template <int P, typename R, int SPLIT>

@@ -55,17 +55,6 @@ __device__ __forceinline__ void flux_n(const R* u, const Prim<R>& w, R nx, R ny,
   F[7] = w.bz * vn - w.vz * bn;
 }
 
-template <typename R>
-__device__ __forceinline__ R fast_speed(const Prim<R>& w, R nx, R ny, R nz, R g) {
-  R ir = R(1) / w.rho;
-  R a2 = g * w.p * ir;
-  R b2 = (w.bx * w.bx + w.by * w.by + w.bz * w.bz) * ir;
-  R bn = w.bx * nx + w.by * ny + w.bz * nz;
-  R bn2 = bn * bn * ir;
-  R s = a2 + b2;
-  return sqrt(R(0.5) * (s + sqrt(fmax(s * s - R(4) * a2 * bn2, R(0)))));
-}
-
 // One side of a face for the HLL flux along the unit normal n: normal velocity and
 // field, total pressure, total enthalpy, v.B and the fast speed, 1/rho formed once.
 template <typename R>
@@ -274,12 +263,6 @@ __device__ __forceinline__ void hlld_acc(const R* uL0, const R* uR0, R nx, R ny,
   }
 #pragma unroll
   for (int v = 0; v < 8; ++v) acc[v] += w * F[v];
-}
-
-template <typename R>
-__device__ __forceinline__ R rusanov_speed(const R* u, R nx, R ny, R nz, R g) {
-  Prim<R> w = to_prim(u, g);
-  return fabs(w.vx * nx + w.vy * ny + w.vz * nz) + fast_speed(w, nx, ny, nz, g);
 }
 
 template <typename R>
