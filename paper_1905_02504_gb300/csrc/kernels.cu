@@ -1976,7 +1976,7 @@ cudaError_t launch_adjoint(const DevTables& T, const DevState& S, const AdjState
   cudaError_t e = launch_adj_ader<P>(T, S, A, dt, st);
   if (e != cudaSuccess) return e;
   k_adj_bperp<P><<<grid_for(T.F), TPB, 0, st>>>(T, S.phi, Wc, A);
-  k_adj_weno<P><<<grid_for(T.Z), TPB, 0, st>>>(T, A);
+  k_adj_weno<P><<<dim3(grid_for(T.Z), 8), TPB, 0, st>>>(T, A);
   return cudaGetLastError();
 }
 template <int P>
@@ -1985,7 +1985,7 @@ cudaError_t launch_adjoint_stage(int stage, const DevTables& T, const DevState& 
   const double* Wc = static_cast<const double*>(S.Wc);
   const double* Bp = static_cast<const double*>(S.Bp);
   switch (stage) {
-    case ST_WENO: k_adj_weno<P><<<grid_for(T.Z), TPB, 0, st>>>(T, A); break;
+    case ST_WENO: k_adj_weno<P><<<dim3(grid_for(T.Z), 8), TPB, 0, st>>>(T, A); break;
     case ST_ADER: return launch_adj_ader<P>(T, S, A, dt, st);
     case ST_FACE: k_adj_face<P><<<grid_for(T.F), TPB, 0, st>>>(T, static_cast<const double*>(S.trF), A, dt); break;
     case ST_EDGE: k_adj_edge<P><<<grid_for(T.E), TPB, 0, st>>>(T, static_cast<const double*>(S.trE), A, dt); break;
