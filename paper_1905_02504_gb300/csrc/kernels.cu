@@ -57,7 +57,9 @@ using namespace dev;
 // as much as any other warp-wide word, so in FP32 one variable per thread is bound by
 // those loads (one per multiply-add).  With VB variables an entry loaded once serves
 // VB multiply-adds (p = 4, 147,456 zones: 275 -> 138 us with VB = 4, 145 us with 2;
-// p = 3, 193,536 zones: 172 -> 93 / 100 us; p = 2, 1,327,104 zones: 474 -> 304 / 279 us).
+// p = 3, 193,536 zones: 172 -> 93 / 100 us).  At p = 2 two variables and eight blocks per
+// SM, which hide the loads' latency, are best (1,327,104 zones: 474 -> 262 us; 322 us with
+// three or four blocks, 273 with seven, 288 with ten).
 // beta_H comes from the upper triangle of the smoothness form (off-diagonals doubled,
 // rows padded to whole 16-byte vectors), and the six face neighbours' differences serve
 // the eight octants that share them.  The FP64 form is bound by its own pipe and keeps
@@ -72,8 +74,8 @@ template <int P> struct WenoVb { static constexpr int VB = P == 2 ? 2 : 4; };
 constexpr long long WENO_WIDE = 20000;
 
 template <int P, typename R, int VB, bool EXACT = false>
-__global__ void __launch_bounds__(TPB, 3) k_weno(const DevTables T, const double* __restrict__ U,
-                                              const float* __restrict__ Uhl, R* __restrict__ Wc) {
+__global__ void __launch_bounds__(TPB, VB == 2 ? 8 : 3) k_weno(const DevTables T, const double* __restrict__ U,
+                                                               const float* __restrict__ Uhl, R* __restrict__ Wc) {
   using Dm = Dim<P>;
   constexpr int NC1 = Dm::NC1, NC1P = Dm::NC1P, SMAX = Dm::SMAX, CH = 16 / sizeof(R);
   const R GH = R(0.85), GK = R(0.15 / 8.0), EPS0 = R(1e-12);
@@ -1168,8 +1170,10 @@ __device__ __forceinline__ void face_flux(const DevTables& T, const R* __restric
   }
 }
 
+// FP32 waits for its trace reads: blocks per SM by measurement (p = 2, 1,327,104 zones,
+// 9 blocks: 309 -> 265 us; p = 3, 193,536 zones, 8: 97 -> 88 us; p = 4, 147,456: 172 -> 150)
 template <int P, typename R, bool HLLD, int SPLIT>
-__global__ void __launch_bounds__(TPB) k_face_flux(const DevTables T, const R* __restrict__ trF,
+__global__ void __launch_bounds__(TPB, sizeof(R) == 4 && !HLLD ? (P == 2 ? 9 : 8) : 1) k_face_flux(const DevTables T, const R* __restrict__ trF,
                                                    double* __restrict__ Ff, double dt) {
   face_flux<P, R, HLLD, SPLIT>(T, trF, Ff, dt, static_cast<long long>(blockIdx.x) * TPB + threadIdx.x);
 }
@@ -1330,8 +1334,10 @@ __device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict
   if (t0 < E * SPLIT && (SPLIT == 1 || t0 % SPLIT == 0)) Ee[e] = dt * G.q * static_cast<double>(acc);
 }
 
+// as for the faces (FP32 p = 2, 10 blocks: 174 -> 153 us; p = 3, 8: 124 -> 109 us; p = 4,
+// 8: 183 -> 171 us)
 template <int P, typename R, int SPLIT>
-__global__ void __launch_bounds__(TPB) k_edge_emf(const DevTables T, const R* __restrict__ trE,
+__global__ void __launch_bounds__(TPB, sizeof(R) == 4 ? (P == 2 ? 10 : 8) : 1) k_edge_emf(const DevTables T, const R* __restrict__ trE,
                                                   double* __restrict__ Ee, double dt) {
   edge_emf<P, R, SPLIT>(T, trE, Ee, dt, static_cast<long long>(blockIdx.x) * TPB + threadIdx.x);
 }
