@@ -104,3 +104,25 @@ def test_cfl_estimate_keeps_the_minimum(kscale, vscale):
         dts.append(m.cfl_dt(0.4) * f)
         m.close()
     assert abs(dts[1] - dts[0]) <= 1e-14 * dts[0]
+
+
+# pressures within 1e-5 of the total energy are out of reach of the FP32 test of the state
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("thermal,flagged", [(1.0, False), (5e-6, False), (-5e-6, True), (-1.0, True)])
+def test_state_flag_near_vacuum(thermal, flagged, prec):
+    from paper_1905_02504_gb300 import geomhd
+    from paper_1905_02504_gb300.inputs import make_problem
+    m = geomhd.Mesh(3, 3, 1.0, 2.0, 2, prec=prec)
+    U, phi = m.initial_state(make_problem("uniform", B0=(0.3, -0.2, 0.5)), nq_zone=3, nq_edge=4)
+    rest = 0.5 * (U[1] ** 2 + U[2] ** 2 + U[3] ** 2) / U[0] + 0.5 * (U[5] ** 2 + U[6] ** 2 + U[7] ** 2)
+    U[4] = rest * (1.0 + abs(thermal))
+    z = m.Z // 2
+    U[4, z] = rest[z] * (1.0 + thermal)
+    m.upload(U, phi)
+    m.step(1e-30)  # too short to change the state
+    if flagged:
+        with pytest.raises(geomhd.GeoError):
+            geomhd.geo_check_state(m.h)
+    else:
+        geomhd.geo_check_state(m.h)
+    m.close()
