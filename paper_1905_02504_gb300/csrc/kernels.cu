@@ -1334,10 +1334,10 @@ __device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict
   if (t0 < E * SPLIT && (SPLIT == 1 || t0 % SPLIT == 0)) Ee[e] = dt * G.q * static_cast<double>(acc);
 }
 
-// as for the faces (FP32 p = 2, 10 blocks: 174 -> 153 us; p = 3, 8: 124 -> 109 us; p = 4,
-// 8: 183 -> 171 us)
+// as for the faces (FP32 p = 2, 10 blocks: 174 -> 153 us; p = 3, 8: 124 -> 109 us); at
+// p = 4 eight blocks help 147,456 zones (183 -> 171 us) and cost 55,296 (80 -> 97 us): left
 template <int P, typename R, int SPLIT>
-__global__ void __launch_bounds__(TPB, sizeof(R) == 4 ? (P == 2 ? 10 : 8) : 1) k_edge_emf(const DevTables T, const R* __restrict__ trE,
+__global__ void __launch_bounds__(TPB, sizeof(R) == 4 && P < 4 ? (P == 2 ? 10 : 8) : 1) k_edge_emf(const DevTables T, const R* __restrict__ trE,
                                                   double* __restrict__ Ee, double dt) {
   edge_emf<P, R, SPLIT>(T, trE, Ee, dt, static_cast<long long>(blockIdx.x) * TPB + threadIdx.x);
 }
