@@ -1482,7 +1482,7 @@ __global__ void __launch_bounds__(TPB) k_update(const DevTables T, double* __res
 }
 
 // ----------------------------------------------------------------------------
-// a8 / a9: CFL time step and div B (deterministic two-pass reductions)
+// a8 / a9: CFL time step (one launch) and div B (two passes), deterministic reductions
 // ----------------------------------------------------------------------------
 constexpr int RED_TPB = 256;
 
@@ -1502,12 +1502,16 @@ __device__ __forceinline__ double warp_max(double v) {
 // result to the caller's pinned host word.  A launch less and no device-to-host copy:
 // 30 -> 19 us a call on small meshes.
 // FP32-bulk meshes first estimate each zone's time step in FP32 from the high parts of
-// the state's split; only zones within 1 % of the warp's smallest estimate so far (the
-// estimate is good to 0.1 %, the pressure's cancellation included) and those whose
-// estimate is not a positive number or has squares near FP32's underflow are evaluated
-// in FP64, so the result is the same
-// and the FP64 square roots and divisions run once or twice per warp instead of for
-// every zone (1,327,104 zones: 213 -> 89 us).
+// the state's split; a zone's own is then evaluated in FP64 if the estimate
+//   - is within 1 % of the warp's smallest so far (it is good to 0.1 %, the pressure's
+//     cancellation included),
+//   - is not a positive number, or is made of numbers near FP32's underflow, or
+//   - does not settle the sign of gamma p + B^2: the sum's rounding errors are below
+//     1e-6 (1 + gamma (gamma - 1)) of |E| + B^2 + m^2 / rho, of which it has to be ten times
+//     as much.
+// So the minimum and what is refused are those of the FP64 form, and the FP64 square
+// roots and divisions run once or twice per warp instead of for every zone (1,327,104
+// zones: 213 -> 89 us).
 __global__ void __launch_bounds__(RED_TPB) k_cfl(const DevTables T, const double* __restrict__ U,
                                                  const float* __restrict__ Uhl, double* __restrict__ part,
                                                  unsigned* __restrict__ ticket, double* __restrict__ out) {
@@ -1531,13 +1535,14 @@ __global__ void __launch_bounds__(RED_TPB) k_cfl(const DevTables T, const double
       const float vx = h[1] * ir, vy = h[2] * ir, vz = h[3] * ir;
       const float b2 = h[5] * h[5] + h[6] * h[6] + h[7] * h[7];
       const float p = (g - 1.f) * ((h[4] - 0.5f * b2) - 0.5f * (h[1] * vx + h[2] * vy + h[3] * vz));
-      const float v2 = vx * vx + vy * vy + vz * vz, c2 = (g * p + b2) * ir;
+      const float v2 = vx * vx + vy * vy + vz * vz, gb = g * p + b2, c2 = gb * ir;
       const float e = static_cast<float>(T.dz0[c]) * static_cast<float>(T.qpow[k]) / (sqrtf(v2) + sqrtf(c2));
       float m = e > 0.f ? e : FLT_MAX;  // a NaN estimate does not hide the others
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
       near = fminf(near, m);
-      look = !(e > 1.01f * near) || !(v2 + c2 > 1e-30f);
+      const float margin = 1e-5f * (g * g) * (fabsf(h[4]) + b2 + h[0] * v2);
+      look = !(e > 1.01f * near && gb > margin && gb > 1e-30f && h[0] > 1e-30f && v2 + c2 > 1e-30f);
     }
     if (look) {
       double u[8];
