@@ -1400,10 +1400,10 @@ __device__ __forceinline__ void update_u(const DevTables& T, double* __restrict_
       Uhl[(8 + v) * Z + z] = static_cast<float>(u[v] - static_cast<double>(hi));
     }
   }
-  // physical-state flag (read by the host between steps)
-  // (p > 0 as (E - B^2 / 2) rho > m^2 / 2, for rho > 0).  In FP32 the difference is good to
-  // 2e-6 of E rho, so a zone that passes by more than 1e-5 of it needs no FP64 test; what
-  // overflows or is not a number does not pass.
+  // Physical-state flag (read by the host between steps): rho > 0, p > 0, E finite.  Most
+  // zones pass without a division, by E rho - (rho B^2 + m^2) / 2 being a clear part of
+  // E rho with all products in range.  FP32 is good to 2e-6 of E rho there, FP64 to 1e-15;
+  // what overflows or is not a number does not pass.  The others get the test itself.
   if (Uhl) {
     float h[8];
 #pragma unroll
@@ -1411,11 +1411,13 @@ __device__ __forceinline__ void update_u(const DevTables& T, double* __restrict_
     const float er = h[4] * h[0];
     const float d = er - 0.5f * (h[0] * (h[5] * h[5] + h[6] * h[6] + h[7] * h[7]) +
                                  (h[1] * h[1] + h[2] * h[2] + h[3] * h[3]));
-    if (h[0] > 0.f && d > 1e-5f * er && er > 1e-30f && er < 1e30f) return;
+    if (d > 1e-5f * er && er > 1e-30f && er < 1e30f && h[0] > 1e-30f && h[4] > 1e-30f) return;
   }
-  const double e = u[4] - 0.5 * (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]);
-  const double m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
-  if (!(u[0] > 0.0) || !(e * u[0] > 0.5 * m2) || !isfinite(u[4])) atomicOr(T.status, 1);
+  const double b2 = u[5] * u[5] + u[6] * u[6] + u[7] * u[7], m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
+  const double er = u[4] * u[0], d = er - 0.5 * (u[0] * b2 + m2);
+  if (d > 1e-10 * er && er > 1e-200 && er < 1e200 && u[0] > 1e-200 && u[4] > 1e-200) return;
+  const double p = pressure_of(u, T.gamma);
+  if (!(u[0] > 0.0) || !(p > 0.0) || !isfinite(u[4])) atomicOr(T.status, 1);
 }
 
 __global__ void __launch_bounds__(TPB) k_split_u(const DevTables T, const double* __restrict__ U,

@@ -51,3 +51,30 @@ def test_cfl_refuses_what_fp32_cannot_tell(part, b):
         assert abs(dts[1] - dts[0]) <= 1e-14 * dts[0]
     for m in meshes:
         m.close()
+
+
+# density, momentum and energy times 4^k and the field times 2^k: the same flow in other
+# units.  At 4^-272 the product of density and energy is below the range of FP64 (so are
+# the squares of the momentum, which is why the unphysical state stops at 4^-200), at 4^250
+# it is near the upper end
+@pytest.mark.parametrize("k,thermal,flagged", [(-272, 1.0, False), (-200, 1.0, False), (0, 1.0, False), (250, 1.0, False),
+                                               (-200, -1e-6, True), (0, -1e-6, True), (250, -1e-6, True)])
+def test_state_flag_in_other_units(k, thermal, flagged):
+    from paper_1905_02504_gb300 import geomhd
+    from paper_1905_02504_gb300.inputs import make_problem
+    m = geomhd.Mesh(3, 3, 1.0, 2.0, 2)
+    U, phi = m.initial_state(make_problem("uniform", B0=(0.3, -0.2, 0.5)), nq_zone=3, nq_edge=4)
+    rest = 0.5 * (U[1] ** 2 + U[2] ** 2 + U[3] ** 2) / U[0] + 0.5 * (U[5] ** 2 + U[6] ** 2 + U[7] ** 2)
+    U[4] = 2.0 * rest
+    U[4, m.Z // 2] = rest[m.Z // 2] * (1.0 + thermal)
+    s = 2.0 ** k
+    U[:5] *= s * s
+    U[5:] *= s
+    m.upload(U, phi * s)
+    m.step(1e-30)  # too short to change the state
+    if flagged:
+        with pytest.raises(geomhd.GeoError):
+            geomhd.geo_check_state(m.h)
+    else:
+        geomhd.geo_check_state(m.h)
+    m.close()
