@@ -227,7 +227,10 @@ int geo_outer_Br2(geo_mesh_t mesh, const double* phi_dev, double* J, double* gph
 
 /* Per-stage device timing, accumulated with CUDA events on the mesh stream while
  * enabled.  ms and counts: arrays of GEO_N_STAGES entries in the order
- * weno, bperp, ader, face_flux, edge_emf, update_u, update_phi (host buffers). */
+ * weno, bperp, ader, face_flux, edge_emf, update_u, update_phi (host buffers).
+ * While it is on, every stage is a launch of its own; with it off, a mesh of at most
+ * 40,000 faces runs its faces and edges in one launch and both updates in another, with
+ * the same result, so that its stage times add up to more than a step. */
 #define GEO_N_STAGES 7
 int geo_set_stage_timing(geo_mesh_t mesh, int enable);
 int geo_get_stage_timing(geo_mesh_t mesh, double* ms, int64_t* counts);

@@ -70,7 +70,9 @@ using namespace dev;
 // between mirror images of a symmetric field) are the ones that its kernels then reverse.
 // ----------------------------------------------------------------------------
 template <int P> struct WenoVb { static constexpr int VB = P == 2 ? 2 : 4; };
-// zones from which the grid with VB variables per thread still fills the GPU
+// zones from which the grid with VB variables per thread fills the GPU (FP32, one variable /
+// VB, us at p = 2, 3, 4: 13,200 zones 12.2 / 12.7, 18.8 / 20.2, 29.0 / 31.4; 18,000 zones
+// 13.0 / 12.7, 26.4 / 21.7, 38.3 / 31.3; 28,512 zones 17.4 / 14.0, 32.6 / 22.8, 48.9 / 32.6)
 constexpr long long WENO_WIDE = 20000;
 
 template <int P, typename R, int VB, bool EXACT = false>
@@ -1097,14 +1099,21 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
 //
 // SPLIT threads (1 or 4 neighbouring lanes) per face take its points in turn and add
 // up their sums.  The FP64 pipe needs 64 cycles of an SM quarter for one instruction
-// of a warp, so a mesh with fewer faces than FACE_SPLIT_MAX, whose warps do not fill
-// the 608 quarters, is as slow as one thread's points in a row; four threads a face
-// cut that chain by four (162 zones at p = 3: 76 -> 24 us), and cost the sums of eight
-// variables over two shuffle steps where the chip is full.
+// of a warp, so a mesh that leaves the 608 quarters with a warp or two each is as slow as
+// one thread's points in a row; four threads a face cut that chain by four (162 zones at
+// p = 3: 76 -> 24 us), and cost the sums of eight variables over two shuffle steps where
+// the chip is full.  Up to SMALL_MESH_FACES faces a step with four threads and the fused
+// launches is the faster one at every order and form, above it the gain is gone within a
+// third more faces (microseconds a step, one thread / four):
+//   faces   p = 2 FP64    p = 3 FP64     p = 4 FP64     p = 2 FP32   p = 3 FP32   p = 4 FP32
+//   23,424   283 / 262     874 /  784    2363 / 2208    65.7 / 54.6   106 /  81    219 / 161
+//   40,200   400 / 375    1313 / 1214    3800 / 3681    69.7 / 63.5   128 / 110    289 / 247
+//   54,600   472 / 484    1631 / 1621    4866 / 4943    71.8 / 69.8   156 / 143    329 / 312
+//   86,400   725 / 724    2588 / 2545    7528 / 7699    85.7 / 86.7   197 / 198    445 / 467
 // The quadrature weight times the Gauss weight is tabulated in the bulk type; the
 // shell's factor q^2k enters once, in FP64.
 // ----------------------------------------------------------------------------
-constexpr long long FACE_SPLIT_MAX = 40000;
+constexpr long long SMALL_MESH_FACES = 40000;
 
 // sum of x over the S neighbouring lanes of a group, in all of them
 template <int S, typename R>
@@ -1172,10 +1181,10 @@ __device__ __forceinline__ void face_flux(const DevTables& T, const R* __restric
 
 // FP32 waits for its trace reads: blocks per SM by measurement (p = 2, 1,327,104 zones,
 // 9 blocks: 309 -> 265 us; p = 3, 193,536 zones, 8: 97 -> 88 us; p = 4, 147,456: 172 -> 150)
-template <int P, typename R, bool HLLD, int SPLIT>
-__global__ void __launch_bounds__(TPB, sizeof(R) == 4 && !HLLD ? (P == 2 ? 9 : 8) : 1) k_face_flux(const DevTables T, const R* __restrict__ trF,
-                                                   double* __restrict__ Ff, double dt) {
-  face_flux<P, R, HLLD, SPLIT>(T, trF, Ff, dt, static_cast<long long>(blockIdx.x) * TPB + threadIdx.x);
+template <int P, typename R, bool HLLD>
+__global__ void __launch_bounds__(TPB, sizeof(R) == 4 && !HLLD ? (P == 2 ? 9 : 8) : 1)
+    k_face_flux(const DevTables T, const R* __restrict__ trF, double* __restrict__ Ff, double dt) {
+  face_flux<P, R, HLLD, 1>(T, trF, Ff, dt, static_cast<long long>(blockIdx.x) * TPB + threadIdx.x);
 }
 
 // ----------------------------------------------------------------------------
@@ -1186,12 +1195,9 @@ __global__ void __launch_bounds__(TPB, sizeof(R) == 4 && !HLLD ? (P == 2 ? 9 : 8
 // boundary edge: one face).  Every index is then static, each zone's sound and Alfven
 // speeds are formed once for its two faces, and no state has to be picked by a runtime
 // index (before: 16 three-way selects per face and point).  SPLIT threads per edge
-// share its points on meshes of fewer than EDGE_SPLIT_MAX edges, as for the faces (162
-// zones at p = 3: 84 -> 25 us).  FP32 p = 4, 147,456 zones: 257 -> 182 us; FP64 p = 4,
-// 110,592 zones: 2.66 -> 2.44 ms.
+// share its points on small meshes, as for the faces (162 zones at p = 3: 84 -> 25 us).
+// FP32 p = 4, 147,456 zones: 257 -> 182 us; FP64 p = 4, 110,592 zones: 2.66 -> 2.44 ms.
 // ----------------------------------------------------------------------------
-constexpr long long EDGE_SPLIT_MAX = 40000;
-
 // the zones and faces around edge e in ring order
 template <int P, typename R>
 struct EdgeRing {
@@ -1336,14 +1342,16 @@ __device__ __forceinline__ void edge_emf(const DevTables& T, const R* __restrict
 
 // as for the faces (FP32 p = 2, 10 blocks: 174 -> 153 us; p = 3, 8: 124 -> 109 us); at
 // p = 4 eight blocks help 147,456 zones (183 -> 171 us) and cost 55,296 (80 -> 97 us): left
-template <int P, typename R, int SPLIT>
-__global__ void __launch_bounds__(TPB, sizeof(R) == 4 && P < 4 ? (P == 2 ? 10 : 8) : 1) k_edge_emf(const DevTables T, const R* __restrict__ trE,
-                                                  double* __restrict__ Ee, double dt) {
-  edge_emf<P, R, SPLIT>(T, trE, Ee, dt, static_cast<long long>(blockIdx.x) * TPB + threadIdx.x);
+template <int P, typename R>
+__global__ void __launch_bounds__(TPB, sizeof(R) == 4 && P < 4 ? (P == 2 ? 10 : 8) : 1)
+    k_edge_emf(const DevTables T, const R* __restrict__ trE, double* __restrict__ Ee, double dt) {
+  edge_emf<P, R, 1>(T, trE, Ee, dt, static_cast<long long>(blockIdx.x) * TPB + threadIdx.x);
 }
 
 // Faces and edges of a small mesh in one launch (blocks below nf: faces): neither alone
-// fills the GPU, and both wait for the predictor only.
+// fills the GPU, and both wait for the predictor only.  A stage run by itself takes the
+// same kernel with the blocks of its half, so that a step in stages (timed ones, the test
+// calls) gives the result of the fused step bit for bit.
 template <int P, typename R, bool HLLD>
 __global__ void __launch_bounds__(TPB) k_face_edge(const DevTables T, const R* __restrict__ trF,
                                                    double* __restrict__ Ff, const R* __restrict__ trE,
@@ -1467,8 +1475,8 @@ __global__ void __launch_bounds__(TPB) k_update_phi(const DevTables T, double* _
   update_phi(T, phi, Ee, f);
 }
 
-// Both updates of a small mesh in one launch (blocks below nz: zones).  The block that
-// draws the last ticket hands the physical-state flag to the host.
+// Both updates of a small mesh in one launch (blocks below nz: zones), or one of them.  The
+// block that draws the last ticket hands the physical-state flag to the host.
 __global__ void __launch_bounds__(TPB) k_update(const DevTables T, double* __restrict__ U,
                                                 const double* __restrict__ Ff, float* __restrict__ Uhl,
                                                 double* __restrict__ phi, const double* __restrict__ Ee,
@@ -1842,6 +1850,24 @@ cudaError_t upload_reference_constants(const Tables& T) {
   return cudaMemcpyToSymbol(RC<P, R>::sym(), &h, sizeof(h));
 }
 
+// what is asked for of a small mesh's faces and edges in one launch, and of its updates in one
+template <int P, typename R>
+void launch_small(const DevTables& T, const DevState& S, double dt, cudaStream_t st, bool faces, bool edges,
+                  bool zones, bool fluxes) {
+  const unsigned nf = faces ? grid_for(4 * T.F) : 0, ne = edges ? grid_for((P == 2 ? 1 : 4) * T.E) : 0;
+  const unsigned nz = zones ? grid_for(T.Z) : 0, np = fluxes ? grid_for(T.F) : 0;
+  const R* trF = static_cast<const R*>(S.trF);
+  const R* trE = static_cast<const R*>(S.trE);
+  if (nf + ne > 0) {
+    if (T.riemann == GEO_RIEMANN_HLLD)
+      k_face_edge<P, R, true><<<nf + ne, TPB, 0, st>>>(T, trF, S.Ff, trE, S.Ee, dt, nf);
+    else
+      k_face_edge<P, R, false><<<nf + ne, TPB, 0, st>>>(T, trF, S.Ff, trE, S.Ee, dt, nf);
+  }
+  if (nz + np > 0)
+    k_update<<<nz + np, TPB, 0, st>>>(T, S.U, S.Ff, S.Uhl, S.phi, S.Ee, S.status_out, S.ticket, nz);
+}
+
 template <int P, typename R>
 cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, double dt, cudaStream_t st) {
   R* Wc = static_cast<R*>(S.Wc);
@@ -1887,28 +1913,24 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
         k_ader<P, R, false><<<grid_for(T.Z), TPB, 0, st>>>(T, S.U, S.phi, Wc, Bp, trF, trE, dt);
       }
       break;
-    case ST_FACE: {
-      auto run = [&](auto hlld) {
-        if (T.F <= FACE_SPLIT_MAX)
-          k_face_flux<P, R, hlld.value, 4><<<grid_for(4 * T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
-        else
-          k_face_flux<P, R, hlld.value, 1><<<grid_for(T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
-      };
-      if (T.riemann == GEO_RIEMANN_HLLD) run(std::true_type{});
-      else run(std::false_type{});
-      break;
-    }
+    case ST_FACE:
     case ST_EDGE:
-      if (P > 2 && T.E <= EDGE_SPLIT_MAX)
-        k_edge_emf<P, R, P == 2 ? 1 : 4><<<grid_for(4 * T.E), TPB, 0, st>>>(T, trE, S.Ee, dt);
-      else
-        k_edge_emf<P, R, 1><<<grid_for(T.E), TPB, 0, st>>>(T, trE, S.Ee, dt);
-      break;
     case ST_UPD_U:
-      k_update_u<<<grid_for(T.Z), TPB, 0, st>>>(T, S.U, S.Ff, S.Uhl);
-      break;
     case ST_UPD_PHI:
-      k_update_phi<<<grid_for(T.F), TPB, 0, st>>>(T, S.phi, S.Ee, S.status_out);
+      if (T.F <= SMALL_MESH_FACES) {
+        launch_small<P, R>(T, S, dt, st, stage == ST_FACE, stage == ST_EDGE, stage == ST_UPD_U, stage == ST_UPD_PHI);
+        break;
+      }
+      if (stage == ST_FACE) {
+        if (T.riemann == GEO_RIEMANN_HLLD) k_face_flux<P, R, true><<<grid_for(T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
+        else k_face_flux<P, R, false><<<grid_for(T.F), TPB, 0, st>>>(T, trF, S.Ff, dt);
+      } else if (stage == ST_EDGE) {
+        k_edge_emf<P, R><<<grid_for(T.E), TPB, 0, st>>>(T, trE, S.Ee, dt);
+      } else if (stage == ST_UPD_U) {
+        k_update_u<<<grid_for(T.Z), TPB, 0, st>>>(T, S.U, S.Ff, S.Uhl);
+      } else {
+        k_update_phi<<<grid_for(T.F), TPB, 0, st>>>(T, S.phi, S.Ee, S.status_out);
+      }
       break;
     default:
       return cudaErrorInvalidValue;
@@ -1917,18 +1939,13 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
 }
 
 // Faces, edges and both updates of a mesh of few faces, in two launches instead of four
-// (162 zones at p = 3: 221 -> 198 us a step; 3,072 zones at p = 2: 173 -> 165 us); false where the mesh is not small.
+// (162 zones at p = 3: 221 -> 198 us a step; 3,072 zones at p = 2: 173 -> 165 us); false
+// where the mesh is not small.
 template <int P, typename R>
 bool launch_corrector_small(const DevTables& T, const DevState& S, double dt, cudaStream_t st, cudaError_t& e) {
-  if (T.F > FACE_SPLIT_MAX) return false;
-  const unsigned nf = grid_for(4 * T.F), ne = grid_for((P == 2 ? 1 : 4) * T.E), nz = grid_for(T.Z);
-  const R* trF = static_cast<const R*>(S.trF);
-  const R* trE = static_cast<const R*>(S.trE);
-  if (T.riemann == GEO_RIEMANN_HLLD)
-    k_face_edge<P, R, true><<<nf + ne, TPB, 0, st>>>(T, trF, S.Ff, trE, S.Ee, dt, nf);
-  else
-    k_face_edge<P, R, false><<<nf + ne, TPB, 0, st>>>(T, trF, S.Ff, trE, S.Ee, dt, nf);
-  k_update<<<nz + grid_for(T.F), TPB, 0, st>>>(T, S.U, S.Ff, S.Uhl, S.phi, S.Ee, S.status_out, S.ticket, nz);
+  if (T.F > SMALL_MESH_FACES) return false;
+  launch_small<P, R>(T, S, dt, st, true, true, false, false);
+  launch_small<P, R>(T, S, dt, st, false, false, true, true);
   e = cudaGetLastError();
   return true;
 }

@@ -126,3 +126,14 @@ def test_state_flag_near_vacuum(thermal, flagged, prec):
     else:
         geomhd.geo_check_state(m.h)
     m.close()
+
+
+# 37,500 faces and 41,256 edges lie on different sides of the size from which one thread
+# takes a whole face or edge: timing the stages must not move a bit of the result
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,nr,p", [(25, 3, 3), (3, 3, 3), (8, 8, 2), (5, 3, 4)])
+def test_stage_timing_leaves_the_result_alone(n, nr, p, prec):
+    U, phi, dt = start(n, nr, 2.0, p)
+    a = one_step(n, nr, 2.0, p, prec, 0, U, phi, dt)
+    b = one_step(n, nr, 2.0, p, prec, 0, U, phi, dt, timing=True)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
