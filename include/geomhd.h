@@ -303,6 +303,8 @@ int geo_time_matrix(int order, double* R, int64_t count);
  * [M-1][NQT][8][Z], 3 predictor states at edge points [M-1][12][NS][8][Z]
  * (buffers 0-3 are FP32 in the FP32-bulk form and are widened to double),
  * 4 time-integrated face fluxes [8][F], 5 time-integrated edge EMFs [E].
+ * 6 the coefficients of buffer 0 as the last geo_step_adjoint recomputed them
+ * (GEO_FP64 meshes; GEO_ERR_STATE before the first).
  * count = number of doubles the host buffer holds; GEO_ERR_ARG if too small.
  * Synchronises the stream. */
 int geo_debug_buffer(geo_mesh_t mesh, int which, double* host, int64_t count);

@@ -235,7 +235,6 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
     }
   }
   D.pinvH = m->upload(PTt, err);
-  D.Qs = m->upload(Qst, err);
   D.oct_nb = m->upload(T.oct_nb, err);
   D.oct_inv = m->upload(T.oct_inv, err);
   D.Q = m->upload(T.Q, err);
@@ -343,7 +342,7 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   std::vector<double> iJF(T.JF.size()), iJE(T.JE.size());
   for (size_t t = 0; t < iJF.size(); ++t) iJF[t] = 1.0 / T.JF[t];
   for (size_t t = 0; t < iJE.size(); ++t) iJE[t] = 1.0 / T.JE[t];
-  D.b64 = geo::BulkTables<double>{D.pinvH, D.oct_inv, D.Q,        D.Qs,      D.TF,       D.nF,       D.wF,
+  D.b64 = geo::BulkTables<double>{D.pinvH, D.oct_inv, D.Q,        nullptr,   D.TF,       D.nF,       D.wF,
                                   D.GB,    D.GM,      D.TN,      D.J0,       D.iJ0,      D.Sm,       D.gcl,
                                   D.JF,    D.JE,      D.se_t,     D.se_nang,  D.se_nradL, D.se_nradR,
                                   m->upload(rfn, err), D.sv_t, m->upload(WFt, err), m->upload(sew, err), m->upload(svw, err),
@@ -712,6 +711,9 @@ int geo_debug_buffer(geo_mesh_t m, int which, double* host, int64_t count) {
     case 3: src = m->ds.trE; n = static_cast<int64_t>(d.M - 1) * 12 * d.NS * 8 * Z; break;
     case 4: src = m->ds.Ff; n = 8 * F; bulk = false; break;
     case 5: src = m->ds.Ee; n = E; bulk = false; break;
+    case 6:
+      if (!m->adj_ready) return fail(GEO_ERR_STATE, "no reverse sweep has run");
+      src = m->adj_fwd.Wc; n = 8LL * d.NC1 * Z; break;
     default: return fail(GEO_ERR_ARG, "unknown buffer");
   }
   if (count < n) return fail(GEO_ERR_ARG, "host buffer too small");
@@ -733,13 +735,6 @@ int geo_debug_buffer(geo_mesh_t m, int which, double* host, int64_t count) {
 
 // one forward stage of the reverse sweep's recompute, on its own buffers
 static cudaError_t adj_forward_stage(geo_mesh* m, int s, double dt) {
-  if (s == geo::ST_WENO) {
-    switch (m->order) {
-      case 2: return geo::launch_weno_exact<2>(m->dt, m->adj_fwd, m->st);
-      case 3: return geo::launch_weno_exact<3>(m->dt, m->adj_fwd, m->st);
-      default: return geo::launch_weno_exact<4>(m->dt, m->adj_fwd, m->st);
-    }
-  }
   switch (m->order) {
     case 2: return geo::launch_stage<2, double>(s, m->dt, m->adj_fwd, dt, m->st);
     case 3: return geo::launch_stage<3, double>(s, m->dt, m->adj_fwd, dt, m->st);

@@ -50,7 +50,7 @@ template <int P, typename R> struct RefConst {
 // threads of a node team read consecutive entries.
 template <typename R> struct BulkTables {
   // pinvH: [ncol][SMAX][NC1P] (coefficients of one stencil zone adjacent, padded to
-  // 16-byte vectors); Qs: upper triangle of Q by rows, off-diagonals doubled, each row
+  // 16-byte vectors); Qs (FP32 only): upper triangle of Q by rows, off-diagonals doubled, each row
   // padded to a multiple of 4 entries
   const R *pinvH, *oct_inv, *Q, *Qs, *TF, *nF, *wF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
   // edge geometry: unit tangents and face normals at the edge points (around a radial
@@ -86,7 +86,7 @@ struct DevTables {
   const int* st_nb;
   const double* pinvH;
   const int* oct_nb;
-  const double *oct_inv, *Q, *Qs, *V0, *l0, *S0, *A0, *TF, *nF, *wF, *WF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
+  const double *oct_inv, *Q, *V0, *l0, *S0, *A0, *TF, *nF, *wF, *WF, *GB, *GM, *TN, *J0, *iJ0, *Sm, *gcl, *JF, *JE;
   const int *col_side_se, *col_side_sgn;
   const int *se_v, *se_col, *se_lf, *se_perm, *se_le, *se_rev;
   const double *se_t, *se_nang, *se_nradL, *se_nradR;
@@ -151,9 +151,6 @@ cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, doubl
 // where the mesh is not small
 template <int P, typename R>
 bool launch_corrector_small(const DevTables& T, const DevState& S, double dt, cudaStream_t st, cudaError_t& e);
-// WENO-AO in the reverse sweep's order of summation (FP64)
-template <int P>
-cudaError_t launch_weno_exact(const DevTables& T, const DevState& S, cudaStream_t st);
 // the FP64 predictor (no positivity) that also stores its Picard
 // iterates for the reverse sweep (It: [P-1][M-1][8][N][Z] doubles)
 template <int P>

@@ -60,14 +60,15 @@ using namespace dev;
 // p = 3, 193,536 zones: 172 -> 93 / 100 us).  At p = 2 two variables and eight blocks per
 // SM, which hide the loads' latency, are best (1,327,104 zones: 474 -> 262 us; 322 us with
 // three or four blocks, 273 with seven, 288 with ten).
-// beta_H comes from the upper triangle of the smoothness form (off-diagonals doubled,
-// rows padded to whole 16-byte vectors), and the six face neighbours' differences serve
-// the eight octants that share them.  The FP64 form is bound by its own pipe and keeps
-// VB = 1, which spreads small meshes over more warps (p = 4, 110,592 zones: 2.02 -> 1.70
-// ms; p = 3, 193,536 zones: 1.99 -> 1.76 ms).
-// EXACT: the order of summation of the reverse sweep's own evaluation (k_adj_weno), bit
-// for bit.  The reverse sweep's recompute takes it, so that its decisions at ties (MinMod
-// between mirror images of a symmetric field) are the ones that its kernels then reverse.
+// The six face neighbours' differences serve the eight octants that share them, and in FP32
+// beta_H comes from the upper triangle of the smoothness form (off-diagonals doubled, rows
+// padded to whole 16-byte vectors).  The FP64 form is bound by its own pipe and keeps VB = 1,
+// which spreads small meshes over more warps, and it keeps the order of summation of the
+// reverse sweep (k_adj_weno): its recompute runs this kernel, so that the branches it
+// reverses are the ones that the step took, also where MinMod meets the mirror images of a
+// symmetric field, which differ by rounding alone.  (The triangular form would save a
+// hundredth of a FP64 step: 110,592 zones at p = 4 28.47 -> 28.18 ms, 193,536 zones at
+// p = 3 16.93 -> 16.76 ms.)
 // ----------------------------------------------------------------------------
 template <int P> struct WenoVb { static constexpr int VB = P == 2 ? 2 : 4; };
 // zones from which the grid with VB variables per thread fills the GPU (FP32, one variable /
@@ -75,11 +76,12 @@ template <int P> struct WenoVb { static constexpr int VB = P == 2 ? 2 : 4; };
 // 13.0 / 12.7, 26.4 / 21.7, 38.3 / 31.3; 28,512 zones 17.4 / 14.0, 32.6 / 22.8, 48.9 / 32.6)
 constexpr long long WENO_WIDE = 20000;
 
-template <int P, typename R, int VB, bool EXACT = false>
+template <int P, typename R, int VB>
 __global__ void __launch_bounds__(TPB, VB == 2 ? 8 : 3) k_weno(const DevTables T, const double* __restrict__ U,
                                                                const float* __restrict__ Uhl, R* __restrict__ Wc) {
   using Dm = Dim<P>;
   constexpr int NC1 = Dm::NC1, NC1P = Dm::NC1P, SMAX = Dm::SMAX, CH = 16 / sizeof(R);
+  constexpr bool FULL = sizeof(R) == 8;
   const R GH = R(0.85), GK = R(0.15 / 8.0), EPS0 = R(1e-12);
   const long long z = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (z >= T.Z) return;
@@ -142,7 +144,7 @@ __global__ void __launch_bounds__(TPB, VB == 2 ? 8 : 3) k_weno(const DevTables T
   R bH[VB];
 #pragma unroll
   for (int v = 0; v < VB; ++v) bH[v] = R(0);
-  if constexpr (!EXACT) {
+  if constexpr (!FULL) {
     const R* q = B.Qs + static_cast<size_t>(c) * Dm::QTRI;
 #pragma unroll
     for (int i = 0; i < NC1; ++i) {
@@ -227,13 +229,13 @@ __global__ void __launch_bounds__(TPB, VB == 2 ? 8 : 3) k_weno(const DevTables T
     fH[v] = wH / GH;
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
-      if constexpr (!EXACT) wK[v][o] = wK[v][o] * itot - fH[v] * GK;
+      if constexpr (!FULL) wK[v][o] = wK[v][o] * itot - fH[v] * GK;
       else wK[v][o] *= itot;
     }
   }
   // out_a = fH (uH_a - GK sum_o uK_oa) + sum_o w_o uK_oa (a < 3), out_m = fH uH_m
   R s3[VB][3];
-  if constexpr (EXACT) {
+  if constexpr (FULL) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       R sk = R(0), wk = R(0);
@@ -1985,15 +1987,6 @@ cudaError_t launch_adj_ader(const DevTables& T, const DevState& S, const AdjStat
   };
   return A.It ? run(k_adj_ader_team<P, true>) : run(k_adj_ader_team<P, false>);
 }
-
-template <int P>
-cudaError_t launch_weno_exact(const DevTables& T, const DevState& S, cudaStream_t st) {
-  k_weno<P, double, 1, true><<<dim3(grid_for(T.Z), 8), TPB, 0, st>>>(T, S.U, nullptr, static_cast<double*>(S.Wc));
-  return cudaGetLastError();
-}
-template cudaError_t launch_weno_exact<2>(const DevTables&, const DevState&, cudaStream_t);
-template cudaError_t launch_weno_exact<3>(const DevTables&, const DevState&, cudaStream_t);
-template cudaError_t launch_weno_exact<4>(const DevTables&, const DevState&, cudaStream_t);
 
 template <int P>
 cudaError_t launch_ader_store_iterates(const DevTables& T, const DevState& S, double* It, double dt, cudaStream_t st) {
