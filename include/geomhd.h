@@ -297,6 +297,13 @@ int geo_prism_derivatives(int order, double* D, int64_t count);
  * host memory with M = order, row 1 zero.  count = doubles the buffer holds. */
 int geo_time_matrix(int order, double* R, int64_t count);
 
+/* The derivative matrices D^alpha of the hexahedral element (Sec. V.c, row i = node,
+ * column j = basis function) as the variable-team predictor and the reverse sweep
+ * apply them, from the element's rings of edges: D [3][N][N] in host memory with
+ * N = 8 / 20 / 32; transposed != 0: from the reverse sweep's transpose, handed
+ * over as D^alpha too.  geo_mesh_create checks both against its tables.  Host only. */
+int geo_ring_derivatives(int order, int transposed, double* D, int64_t count);
+
 /* Copy one internal work buffer of the last step to host memory, for stage-by-
  * stage verification: which = 0 WENO-AO Taylor coefficients [8][NC1][Z],
  * 1 nodal normal B per face [NQmax][F], 2 predictor states at face points

@@ -169,37 +169,63 @@ __device__ __forceinline__ void ring_nodes(const R* row, int q, R* edge, R* inne
   }
 }
 
-// derivative along one axis of a lane's edge nodes f[0..P) and, with the two ring
-// edges of its face, of the face's perpendicular inner nodes f[P..K); in place
+// Derivative along one axis of a lane's edge nodes f[0..P) and, with the two ring
+// edges of its face, of the face's perpendicular inner nodes f[P..K).  RingEdge: what a lane
+// forms from its own edge, a and b of which the lane of ring edge q - 1 needs as well
+// (host code too: ring_matrix checks the coefficients against the element's D^alpha).
+template <typename R>
+struct RingEdge {
+  R u, a, b;
+};
 template <int P, typename R>
-__device__ __forceinline__ void ring_derivative(R* f, int lane) {
-  const int next = (lane + 8) & 31;  // the same variable of ring edge q + 1
+__host__ __device__ __forceinline__ RingEdge<R> ring_edge(const R* f) {
+  RingEdge<R> e{R(0), R(0), R(0)};
   if constexpr (P == 2) {
-    f[0] = f[1] - f[0];
-    f[1] = f[0];
+    e.u = f[1] - f[0];
   } else if constexpr (P == 3) {
-    const R d = f[2] - f[0], g = (f[0] + f[2]) - R(2) * f[1];
-    const R G = g + __shfl_sync(0xffffffffu, g, next);
+    e.u = f[2] - f[0];
+    e.a = (f[0] + f[2]) - R(2) * f[1];
+  } else {
+    const R u = f[3] - f[0], g = (f[0] + f[3]) - (f[1] + f[2]), r = u - R(3) * (f[2] - f[1]);
+    e.u = u;
+    e.a = r + g;
+    e.b = r - g;
+  }
+  return e;
+}
+template <int P, typename R>
+__host__ __device__ __forceinline__ void ring_apply(R* f, const RingEdge<R>& e, R an, R bn) {
+  if constexpr (P == 2) {
+    f[0] = e.u;
+    f[1] = e.u;
+  } else if constexpr (P == 3) {
+    const R G = e.a + an;
     const R t = f[4] - f[3];
-    f[0] = d - R(2) * g;
-    f[1] = d;
-    f[2] = d + R(2) * g;
+    f[0] = e.u - R(2) * e.a;
+    f[1] = e.u;
+    f[2] = e.u + R(2) * e.a;
     f[3] = t - G;
     f[4] = t + G;
   } else {
-    const R u = f[3] - f[0], g = (f[0] + f[3]) - (f[1] + f[2]), r = u - R(3) * (f[2] - f[1]);
-    const R A = r + g, B = r - g;
-    const R An = __shfl_sync(0xffffffffu, A, next), Bn = __shfl_sync(0xffffffffu, B, next);
     const R t1 = f[6] - f[4], t2 = f[7] - f[5];
-    f[0] = u + R(2.25) * B;
-    f[1] = u - R(0.75) * A;
-    f[2] = u - R(0.75) * B;
-    f[3] = u + R(2.25) * A;
-    f[4] = (t1 + R(1.5) * B) + R(0.75) * Bn;
-    f[5] = (t2 + R(0.75) * B) + R(1.5) * Bn;
-    f[6] = (t1 + R(1.5) * A) + R(0.75) * An;
-    f[7] = (t2 + R(0.75) * A) + R(1.5) * An;
+    f[0] = e.u + R(2.25) * e.b;
+    f[1] = e.u - R(0.75) * e.a;
+    f[2] = e.u - R(0.75) * e.b;
+    f[3] = e.u + R(2.25) * e.a;
+    f[4] = (t1 + R(1.5) * e.b) + R(0.75) * bn;
+    f[5] = (t2 + R(0.75) * e.b) + R(1.5) * bn;
+    f[6] = (t1 + R(1.5) * e.a) + R(0.75) * an;
+    f[7] = (t2 + R(0.75) * e.a) + R(1.5) * an;
   }
+}
+template <int P, typename R>
+__device__ __forceinline__ void ring_derivative(R* f, int lane) {
+  const int next = (lane + 8) & 31;  // the same variable of ring edge q + 1
+  const RingEdge<R> e = ring_edge<P>(f);
+  R an = R(0), bn = R(0);
+  if constexpr (P > 2) an = __shfl_sync(0xffffffffu, e.a, next);
+  if constexpr (P == 4) bn = __shfl_sync(0xffffffffu, e.b, next);
+  ring_apply<P>(f, e, an, bn);
 }
 
 // contraction of one zone by its warp: F rows in, dF entries out, in place

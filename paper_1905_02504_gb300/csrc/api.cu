@@ -984,6 +984,14 @@ int geo_time_matrix(int order, double* R, int64_t count) {
   return GEO_OK;
 }
 
+int geo_ring_derivatives(int order, int transposed, double* D, int64_t count) {
+  if (order < 2 || order > 4 || !D) return fail(GEO_ERR_ARG, "geo_ring_derivatives: bad arguments");
+  const int64_t n = order == 2 ? 8 : (order == 3 ? 20 : 32);
+  if (count < 3 * n * n) return fail(GEO_ERR_ARG, "geo_ring_derivatives: host buffer too small");
+  for (int a = 0; a < 3; ++a) geo::ring_matrix_any(order, a, transposed != 0, D + a * n * n);
+  return GEO_OK;
+}
+
 int geo_prism_derivatives(int order, double* D, int64_t count) {
   if (order < 2 || order > 4 || !D) return fail(GEO_ERR_ARG, "geo_prism_derivatives: bad arguments");
   std::vector<double> n, d;

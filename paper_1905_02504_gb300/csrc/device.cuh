@@ -144,6 +144,9 @@ struct Tables;
 template <int P, typename R>
 cudaError_t upload_reference_constants(const Tables& T);
 
+// D^axis as the ring kernels apply it (kernels.cu), [N][N] at the order p; returns N
+int ring_matrix_any(int p, int axis, bool transposed, double* D);
+
 // launchers (kernels.cu); return cudaGetLastError() of the launch
 template <int P, typename R>
 cudaError_t launch_stage(int stage, const DevTables& T, const DevState& S, double dt, cudaStream_t st);

@@ -1719,9 +1719,37 @@ int reduction_blocks(long long n) {
   return static_cast<int>(b);
 }
 
+// D^axis [N][N] as the ring kernels apply it, column by column: the derivative of each
+// node's basis function, or (transposed) the transpose of the reverse sweep's form
+template <int P>
+void ring_matrix(int axis, bool transposed, double* D) {
+  using G = Ring<P>;
+  constexpr int N = Dim<P>::N;
+  for (int j = 0; j < N; ++j) {
+    double f[4][G::K];
+    for (int q = 0; q < 4; ++q)
+      for (int k = 0; k < G::K; ++k) f[q][k] = G::node(axis, q, k) == j ? 1.0 : 0.0;
+    if (!transposed) {
+      RingEdge<double> e[4];
+      for (int q = 0; q < 4; ++q) e[q] = ring_edge<P>(f[q]);
+      for (int q = 0; q < 4; ++q) ring_apply<P>(f[q], e[q], e[(q + 1) & 3].a, e[(q + 1) & 3].b);
+    } else {
+      double a[4], b[4];
+      for (int q = 0; q < 4; ++q) ring_edge_t<P>(f[q], a[q], b[q]);
+      for (int q = 0; q < 4; ++q) ring_apply_t<P>(f[q], a[q], a[(q + 3) & 3], b[(q + 3) & 3]);
+    }
+    for (int q = 0; q < 4; ++q)
+      for (int k = 0; k < G::K; ++k) {
+        const int i = G::node(axis, q, k);
+        D[transposed ? j * N + i : i * N + j] = f[q][k];
+      }
+  }
+}
+
 // Places and weights of the ring order.  The kernels use one set of point weights
 // for all faces and edges, so every face's and edge's own weights are checked
-// against it, node by node; false if the element does not have that symmetry.
+// against it, node by node, and the rings' derivatives and their transposes against
+// D^alpha; false if the element does not have that symmetry.
 template <int P, typename R>
 bool ring_constants(const Tables& T, RefConst<P, R>& h) {
   using Dm = Dim<P>;
@@ -1738,6 +1766,13 @@ bool ring_constants(const Tables& T, RefConst<P, R>& h) {
   }
   double tab[3][Dm::NQS * NFN + 3 * NFN] = {};
   auto same = [](double a, double b) { return std::fabs(a - b) <= 1e-12; };
+  for (int a = 0; a < 3; ++a)
+    for (int t = 0; t < 2; ++t) {
+      double D[N * N];
+      ring_matrix<P>(a, t == 1, D);
+      for (int e = 0; e < N * N; ++e)
+        if (std::fabs(D[e] - T.D[static_cast<size_t>(a) * N * N + e]) > 1e-10) return false;
+    }
   const int lf_of_q[4] = {2, 1, 3, 0};
   for (int q = 0; q < 4; ++q) {
     int nd[NFN];
@@ -1950,6 +1985,13 @@ bool launch_corrector_small(const DevTables& T, const DevState& S, double dt, cu
   launch_small<P, R>(T, S, dt, st, false, false, true, true);
   e = cudaGetLastError();
   return true;
+}
+
+int ring_matrix_any(int p, int axis, bool transposed, double* D) {
+  if (p == 2) ring_matrix<2>(axis, transposed, D);
+  else if (p == 3) ring_matrix<3>(axis, transposed, D);
+  else ring_matrix<4>(axis, transposed, D);
+  return p == 2 ? Dim<2>::N : (p == 3 ? Dim<3>::N : Dim<4>::N);
 }
 
 #define GEO_INSTANTIATE(P, R)                                                                       \

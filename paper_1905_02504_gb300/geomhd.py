@@ -64,6 +64,7 @@ _SIGS = {
     "geo_prism_predictor": [ctypes.c_int, _i64, _vp, _vp, _d, _d, _vp, _vp],
     "geo_prism_nodes": [ctypes.c_int, _vp, _i64],
     "geo_prism_derivatives": [ctypes.c_int, _vp, _i64],
+    "geo_ring_derivatives": [ctypes.c_int, ctypes.c_int, _vp, _i64],
     "geo_time_matrix": [ctypes.c_int, _vp, _i64],
     "geo_host_geometry": [ctypes.c_int, ctypes.c_int, _d, _d, ctypes.c_int, _i64, _i64, _vp, _vp, _vp, _vp],
     "geo_debug_buffer": [_h, ctypes.c_int, _vp, _i64],
@@ -287,6 +288,14 @@ def geo_prism_derivatives(order):
     n = {2: 6, 3: 15, 4: 26}[order]
     out = np.empty((3, n, n))
     _check(_lib.geo_prism_derivatives(order, _ptr(out), out.size), "geo_prism_derivatives")
+    return out
+
+
+def geo_ring_derivatives(order, transposed=False):
+    """The hexahedron's D^alpha as the ring kernels apply it, (3, N, N)."""
+    n = {2: 8, 3: 20, 4: 32}[order]
+    out = np.empty((3, n, n))
+    _check(_lib.geo_ring_derivatives(order, int(transposed), _ptr(out), out.size), "geo_ring_derivatives")
     return out
 
 

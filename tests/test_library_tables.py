@@ -43,3 +43,16 @@ def test_library_geometry_matches_oracle_on_cpu(n, nr, p):
     assert np.abs(nrm - ref_n).max() <= 1e-13 * ref_a.max()
     close = (om.zone_face_sign[..., None] * nrm[om.zone_face]).sum(1)
     assert np.abs(close).max() <= 1e-14 * ref_a.max()
+
+
+@pytest.mark.parametrize("transposed", [False, True])
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_ring_derivatives_are_the_elements(p, transposed):
+    """The predictor's contraction on the rings of edges, and its transpose in the reverse
+    sweep, are the oracle element's D^alpha (their coefficients are written in the kernels)."""
+    from oracle import refelem
+    from paper_1905_02504_gb300 import geomhd
+    D = refelem.HexElement(p).D
+    R = geomhd.geo_ring_derivatives(p, transposed)
+    for a in range(3):
+        assert np.abs(R[a] - D[a]).max() <= 1e-12 * np.abs(D[a]).max()
