@@ -57,3 +57,26 @@ def test_generated_header_is_current(tmp_path):
     assert text == refpattern.header()
     for p, nnz in ((2, 16), (3, 96), (4, 192)):
         assert "struct RefPattern<%d>" % p in text and "NNZ = %d," % nnz in text
+
+
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_triangle_derivatives_are_the_prisms(p):
+    """The compiled derivatives of the triangular element along its edges 0-1 and 0-2 are the
+    oracle prism's on each triangular face (nodes in the prism's order), and nothing else
+    of the prism enters there."""
+    from oracle import prism
+    el = prism.PrismElement(p)
+    tri = refpattern.triangle_nodes(p)
+    dirs = [prism.TRI[1] - prism.TRI[0], prism.TRI[2] - prism.TRI[0]]
+    for zeta in (0.5, -0.5):
+        face = []
+        for s, t in tri:
+            x = prism.TRI[0] + float(s) * dirs[0] + float(t) * dirs[1]
+            face.append(int(np.argmin(np.abs(el.nodes - np.array([x[0], x[1], zeta])).sum(1))))
+        assert len(set(face)) == len(face)
+        for d, ent in zip(dirs, refpattern.triangle_derivatives(p)):
+            full = d[0] * el.D[0] + d[1] * el.D[1]
+            T = np.zeros((len(face), el.N))
+            for i, j, v in ent:
+                T[i, face[j]] = float(v)
+            assert np.abs(full[face] - T).max() <= 1e-12 * np.abs(full).max()
