@@ -6,6 +6,8 @@ import os
 import subprocess
 import sys
 
+import pytest
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 ARGS = ["--impl", "reference", "--steps", "1", "--warmup", "0", "--sample-n", "2", "--sample-nr", "2",
         "--order", "2"]
@@ -35,3 +37,43 @@ def test_reference_arm_two_ranks_prints_once():
     assert r.returncode == 0, r.stderr[-2000:]
     lines = json_lines(r.stdout)
     assert len(lines) == 1 and lines[0]["n_gpus"] == 2
+
+
+@pytest.mark.parametrize("p,n,nnz,nedge", [(2, 8, 16, 1), (3, 20, 96, 2), (4, 32, 192, 3)])
+def test_roofline_counts_what_the_predictor_executes(p, n, nnz, nedge):
+    """The roofline's operations are those of the kernel that ran: for the ring predictor the
+    operations of its contraction (counted here by running its formulas on numbers that
+    count), not the sparse rows' of geo_stage_flops, with which it came out above the peak."""
+    import bench
+
+    class Num:
+        ops = 0
+
+        def __add__(self, o):
+            Num.ops += 1
+            return Num()
+        __sub__ = __mul__ = __rmul__ = __add__
+
+    x = [Num() for _ in range(8)]
+    if p == 2:
+        x[1] - x[0]
+        Num.ops *= 2  # each end takes the difference itself
+    elif p == 3:
+        d, g = x[2] - x[0], (x[0] + x[2]) - 2.0 * x[1]
+        G, t = g + x[5], x[4] - x[3]
+        d - 2.0 * g, d + 2.0 * g, t - G, t + G
+    else:
+        u, g = x[3] - x[0], (x[0] + x[3]) - (x[1] + x[2])
+        r = u - 3.0 * (x[2] - x[1])
+        A, B, t1, t2 = r + g, r - g, x[6] - x[4], x[7] - x[5]
+        u + 2.25 * B, u - 0.75 * A, u - 0.75 * B, u + 2.25 * A
+        for t, y in ((t1, B), (t2, B), (t1, A), (t2, A)):
+            (t + 1.5 * y) + 0.75 * x[0]
+    ring = 4 * Num.ops + n          # four ring edges, then a sum at every node
+    levels = 1 + (p - 1) * (p - 1)
+    points = (p - 1) * 12 * (nedge - 1) * 4 * 16 if p == 4 else 0
+    counted = 1e6
+    got = bench.executed_flops(counted, "ader", bench.kernel_name("ader", None, False, p), p)
+    assert got == counted - levels * 24 * (2 * nnz - ring) - points
+    assert bench.executed_flops(counted, "ader", "k_ader_team", p) == counted
+    assert bench.executed_flops(counted, "weno", "k_weno", p) == counted
