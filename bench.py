@@ -99,9 +99,7 @@ def workload_name(a):
         6, a.n, a.n, a.nr, 6 * a.n * a.n * a.nr, a.order, form, getattr(a, "problem", "smooth"), extra)
 
 
-def default_schedule(order, fp32=False):
-    """The library's default predictor schedule: the variable team."""
-    return 2
+DEFAULT_SCHEDULE = 2  # the library's default predictor schedule: the variable team
 
 
 def kernel_name(stage, pred, positivity=False, order=4, fp32=False):
@@ -111,7 +109,7 @@ def kernel_name(stage, pred, positivity=False, order=4, fp32=False):
     name = "k_" + stage
     if stage == "ader":
         if pred is None:
-            pred = default_schedule(order, fp32)
+            pred = DEFAULT_SCHEDULE
         if pred == 2 and (not positivity or order == 4 or (order == 3 and not fp32)):
             name += "_ring"
         elif pred != 0:
@@ -135,10 +133,10 @@ def executed_flops(counted, stage, kernel, order):
     return counted - saved
 
 
-def sched_name(pred, order, fp32=False):
+def sched_name(pred):
     """Predictor schedule in use."""
     if pred is None:
-        pred = default_schedule(order, fp32)
+        pred = DEFAULT_SCHEDULE
     return {0: "zone-thread", 1: "node-team", 2: "variable-team"}[pred]
 
 
@@ -416,7 +414,7 @@ def fp32_bulk_leg(a, mesh64, U0, phi0, dt, stream, flush, barrier, ws):
         "stages": {geomhd.STAGES[s]: {"avg_ms": float(avg[s]), "share": float(stage_ms[s] / stage_ms.sum())}
                    for s in range(geomhd.N_STAGES)},
         "rel_l1_vs_fp64": err, "rel_l1_phi_vs_fp64": errp, "steps_compared": a.compare_steps,
-        "predictor": sched_name(a.predictor, a.order, True),
+        "predictor": sched_name(a.predictor),
         "divB_rel": r32,
     }
     m32.close()
@@ -575,7 +573,7 @@ def gpu_arm(a):
             "data": "synthetic",
             "config": {"workload": workload_name(a), "zones": Z, "order": a.order, "dt": dt,
                        "problem": a.problem, "positivity": a.positivity,
-                       "predictor": sched_name(a.predictor, a.order, a.fp32_only),
+                       "predictor": sched_name(a.predictor),
                        "cfl": a.cfl, "l2": "flushed between steps (512 MB write)",
                        "parallelism": "replicas" if ws > 1 else "single GPU"},
             # per step: the seven stage kernels, the trace positivity kernel when the
@@ -773,9 +771,10 @@ def convergence_arm(a):
 def contraction_arm(a):
     """The predictor's contraction sum_alpha D^alpha F^alpha (Eq. C.34) timed alone,
     as many times per zone as the FP32-bulk predictor performs it (level 1, then
-    p Picard iterations over levels 2..M), in the CUDA-core form of the variable
-    team and in a tensor-core form (mma.sync TF32, three passes), beside the
-    predictor kernel's own time per step on the same mesh."""
+    p Picard iterations over levels 2..M), in a CUDA-core form on the sparse rows of
+    D^alpha and in a tensor-core form (mma.sync TF32, three passes), beside the time
+    per step of the predictor kernel on the same mesh (which contracts in another form,
+    with fewer operations)."""
     import numpy as np
     import torch
     from paper_1905_02504_gb300 import geomhd
@@ -786,7 +785,7 @@ def contraction_arm(a):
     a.fp32_only = True
     mesh = geomhd.Mesh(a.n, a.nr, *domain(a.problem), p, prec=geomhd.GEO_FP32_BULK, stream=stream.cuda_stream,
                        gamma=make_problem(a.problem).gamma)
-    pred = default_schedule(p, True) if a.predictor is None else a.predictor
+    pred = DEFAULT_SCHEDULE if a.predictor is None else a.predictor
     geomhd.geo_set_predictor(mesh.h, pred)
     U0, phi0 = mesh.initial_state(make_problem(a.problem))
     mesh.upload(U0, phi0)
@@ -813,13 +812,12 @@ def contraction_arm(a):
         ms = [geomhd.geo_probe_contraction(mesh.h, tensor, Z, reps, out) for _ in range(3)]
         t = float(np.median(ms))
         useful = 2.0 * 3 * nnz * 8 * reps * Z
-        forms[name] = {"ms": round(t, 4), "share_of_predictor": round(t / pred_ms, 3),
-                       "useful_tflops": round(useful / (t * 1e-3) / 1e12, 2)}
+        forms[name] = {"ms": round(t, 4), "useful_tflops": round(useful / (t * 1e-3) / 1e12, 2)}
     mp, kp = (N + 15) // 16 * 16, (3 * N + 7) // 8 * 8
     forms["mma_sync_tf32x3_dense"]["issued_tflops"] = round(
         3 * 2.0 * mp * kp * 8 * reps * Z / (forms["mma_sync_tf32x3_dense"]["ms"] * 1e-3) / 1e12, 1)
     print(json.dumps({"study": "predictor contraction alone, FP32", "workload": workload_name(a), "order": p,
-                      "zones": Z, "contractions_per_zone": reps, "predictor_schedule": sched_name(pred, p, True),
+                      "zones": Z, "contractions_per_zone": reps, "predictor_schedule": sched_name(pred),
                       "predictor_ms_per_step": round(pred_ms, 4), "forms": forms}), flush=True)
     mesh.close()
 

@@ -248,9 +248,9 @@ int geo_probe_fma_peak(int prec, void* stream, double* flops_per_s);
 
 /* Measurement probe of the predictor's derivative contraction (Eq. C.34,
  * dF_{v,i} = sum_alpha sum_j D^alpha_ij F^alpha_{v,j}) alone, FP32, on the mesh's
- * order: tensor = 0 times the CUDA-core sparse form of the variable-team
- * predictor, tensor = 1 a tensor-core form (mma.sync TF32, three-pass split,
- * dense padded D).  F of each zone is a fixed hash of (zone, alpha, v, j) made on
+ * order: tensor = 0 times a CUDA-core form on the sparse rows of D^alpha, tensor = 1
+ * a tensor-core form (mma.sync TF32, three-pass split, dense padded D).  F of each
+ * zone is a fixed hash of (zone, alpha, v, j) made on
  * the device (no HBM reads); the contraction runs `reps` times per zone over
  * `zones` zones and the last result goes to out_dev (device, zones x 8 x N
  * floats, [zone][v][node], caller-owned).  *ms = duration of one launch (CUDA

@@ -26,8 +26,9 @@
 // warp, so the exchange needs no block barrier; without, nodes are packed densely
 // over the block's threads (P = 2, 3) and the exchanges are block barriers.
 //
-// Bounds.  FP64: the FP64 pipe (fewer operations are the gain).  FP32: the shared
-// memory data path (64-68 % busy at p = 3, 4) and instruction issue (53-63 %) together.
+// Bounds (196,608 zones).  FP64: the FP64 pipe, 89 % busy at every order (fewer operations
+// are the gain).  FP32: the shared memory data path and instruction issue together, 79 %
+// and 65 % busy at p = 3, 69 % and 53 % at p = 4, 73 % and 71 % at p = 2.
 // Measured, predictor alone, against the sparse rows on the compiled pattern of D^alpha
 // (FP64 p = 4: the node team's padded rows):
 //   FP32 p = 4, 147,456 zones  2446 -> 1288 us     FP64 p = 4, 110,592 zones  26.98 -> 20.95 ms
@@ -83,12 +84,30 @@ struct Ring {
 // lane = node.  P = 3: a warp holds four nodes of the block's eight zones (zone
 // fastest); P = 2: eight nodes of four zones.
 template <int P, typename R> struct RingCfg;
-template <> struct RingCfg<2, float> { static constexpr bool POS = false, WARP = false; static constexpr int ZB = 16, MINB = 14; };
-template <> struct RingCfg<3, float> { static constexpr bool POS = false, WARP = false; static constexpr int ZB = 8, MINB = 7; };
-template <> struct RingCfg<4, float> { static constexpr bool POS = true, WARP = true; static constexpr int ZB = 4, MINB = 5; };
-template <> struct RingCfg<2, double> { static constexpr bool POS = false, WARP = false; static constexpr int ZB = 16, MINB = 4; };
-template <> struct RingCfg<3, double> { static constexpr bool POS = true, WARP = false; static constexpr int ZB = 8, MINB = 3; };
-template <> struct RingCfg<4, double> { static constexpr bool POS = true, WARP = true; static constexpr int ZB = 4, MINB = 2; };
+template <> struct RingCfg<2, float> {
+  static constexpr bool POS = false, WARP = false;
+  static constexpr int ZB = 16, MINB = 14;
+};
+template <> struct RingCfg<3, float> {
+  static constexpr bool POS = false, WARP = false;
+  static constexpr int ZB = 8, MINB = 7;
+};
+template <> struct RingCfg<4, float> {
+  static constexpr bool POS = true, WARP = true;
+  static constexpr int ZB = 4, MINB = 5;
+};
+template <> struct RingCfg<2, double> {
+  static constexpr bool POS = false, WARP = false;
+  static constexpr int ZB = 16, MINB = 4;
+};
+template <> struct RingCfg<3, double> {
+  static constexpr bool POS = true, WARP = false;
+  static constexpr int ZB = 8, MINB = 3;
+};
+template <> struct RingCfg<4, double> {
+  static constexpr bool POS = true, WARP = true;
+  static constexpr int ZB = 4, MINB = 2;
+};
 
 template <int P, typename R>
 struct RingLayout {
@@ -550,7 +569,8 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
 #pragma unroll
             for (int t = 0; t < ZB; ++t) s[t] += gb * x[t];
           }
-          for (int t = z0; t < z1; ++t) S.F[t * L::FZ + (5 + warp) * L::RS + i] = t == 0 ? s[0] : (t == 1 ? s[1] : (t == 2 ? s[2] : s[3]));
+          for (int t = z0; t < z1; ++t)
+            S.F[t * L::FZ + (5 + warp) * L::RS + i] = t == 0 ? s[0] : (t == 1 ? s[1] : (t == 2 ? s[2] : s[3]));
         } else {
           const R* TN = BT.TN + static_cast<size_t>(cc) * N * NC1 + i;
           R s[5][ZB];
@@ -825,7 +845,8 @@ __global__ void __launch_bounds__(RingLayout<P, R>::NT, RingCfg<P, R>::MINB)
       const R w = __ldg(iJ + idx);
       R* o = out + at + static_cast<size_t>(static_cast<unsigned>(idx)) * Z8;
 #pragma unroll
-      for (int m = 0; m < static_cast<int>(sizeof(s) / sizeof(R)); ++m) emit(in && mine, s[m] * w, o + (m0 + m) * step + off);
+      for (int m = 0; m < static_cast<int>(sizeof(s) / sizeof(R)); ++m)
+        emit(in && mine, s[m] * w, o + (m0 + m) * step + off);
     };
     const R* row = S.F + zt * L::FL + v * L::RS;
     ring_points<P, ML, POS>(

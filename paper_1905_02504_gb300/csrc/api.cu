@@ -222,15 +222,18 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   const int nc1p = (d.NC1 + 3) / 4 * 4;
   int qtri = 0;
   for (int i = 0; i < d.NC1; ++i) qtri += (d.NC1 - i + 3) / 4 * 4;
-  std::vector<double> PTt(static_cast<size_t>(T.ncol) * d.SMAX * nc1p, 0.0), Qst(static_cast<size_t>(T.ncol) * qtri, 0.0);
+  std::vector<double> PTt(static_cast<size_t>(T.ncol) * d.SMAX * nc1p, 0.0);
+  std::vector<double> Qst(prec == GEO_FP32_BULK ? static_cast<size_t>(T.ncol) * qtri : 0, 0.0);
   for (int c = 0; c < T.ncol; ++c) {
+    const double* pinv = &T.pinvH[static_cast<size_t>(c) * d.NC1 * d.SMAX];
     for (int j = 0; j < d.SMAX; ++j)
-      for (int i = 0; i < d.NC1; ++i)
-        PTt[(static_cast<size_t>(c) * d.SMAX + j) * nc1p + i] = T.pinvH[(static_cast<size_t>(c) * d.NC1 + i) * d.SMAX + j];
+      for (int i = 0; i < d.NC1; ++i) PTt[(static_cast<size_t>(c) * d.SMAX + j) * nc1p + i] = pinv[i * d.SMAX + j];
+    if (Qst.empty()) continue;
     size_t at = static_cast<size_t>(c) * qtri;
+    const double* Qc = &T.Q[static_cast<size_t>(c) * d.NC1 * d.NC1];
     for (int i = 0; i < d.NC1; ++i) {
-      const double* Qc = &T.Q[static_cast<size_t>(c) * d.NC1 * d.NC1];
-      for (int j = i; j < d.NC1; ++j) Qst[at + j - i] = i == j ? Qc[i * d.NC1 + i] : Qc[i * d.NC1 + j] + Qc[j * d.NC1 + i];
+      Qst[at] = Qc[i * d.NC1 + i];
+      for (int j = i + 1; j < d.NC1; ++j) Qst[at + j - i] = Qc[i * d.NC1 + j] + Qc[j * d.NC1 + i];
       at += (d.NC1 - i + 3) / 4 * 4;
     }
   }
@@ -255,11 +258,13 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
     const size_t g0 = static_cast<size_t>(c) * NR * d.NBIN, t0 = static_cast<size_t>(c) * d.N * d.NC1;
     const size_t cb = static_cast<size_t>(c) * d.NBIN;
     for (int b = 0; b < d.NBIN; ++b) {
-      for (int r = 0; r < 3; ++r) GMt[3 * cb + static_cast<size_t>(r) * d.NBIN + b] = T.GB[g0 + static_cast<size_t>(r) * d.NBIN + b];
-      for (int r = 3; r < NR; ++r) GBt[(cb + b) * (NR - 3) + r - 3] = T.GB[g0 + static_cast<size_t>(r) * d.NBIN + b];
+      auto gb = [&](int r) { return T.GB[g0 + static_cast<size_t>(r) * d.NBIN + b]; };
+      for (int r = 0; r < 3; ++r) GMt[3 * cb + static_cast<size_t>(r) * d.NBIN + b] = gb(r);
+      for (int r = 3; r < NR; ++r) GBt[(cb + b) * (NR - 3) + r - 3] = gb(r);
     }
     for (int i = 0; i < d.N; ++i)
-      for (int mm = 0; mm < d.NC1; ++mm) TNt[t0 + static_cast<size_t>(mm) * d.N + i] = T.TN[t0 + static_cast<size_t>(i) * d.NC1 + mm];
+      for (int mm = 0; mm < d.NC1; ++mm)
+        TNt[t0 + static_cast<size_t>(mm) * d.N + i] = T.TN[t0 + static_cast<size_t>(i) * d.NC1 + mm];
   }
   D.GB = m->upload(GBt, err);
   D.GM = m->upload(GMt, err);
@@ -308,8 +313,8 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
       }
       used[f] = true;
       const double sg = fL[f] == at ? 1.0 : -1.0;
-      for (int t = 0; t < NS * 3; ++t)
-        rfn[(static_cast<size_t>(4) * sv + j) * NS * 3 + t] = sg * T.sv_fn[(static_cast<size_t>(4) * sv + f) * NS * 3 + t];
+      const double* nv = &T.sv_fn[(static_cast<size_t>(4) * sv + f) * NS * 3];
+      for (int t = 0; t < NS * 3; ++t) rfn[(static_cast<size_t>(4) * sv + j) * NS * 3 + t] = sg * nv[t];
       at = fL[f] == at ? fR[f] : fL[f];
     }
     if (at != 0) err = cudaErrorInvalidValue;  // the ring must close
@@ -345,8 +350,8 @@ int geo_mesh_create(int subdiv, int nr, double r_in, double r_out, int order, in
   D.b64 = geo::BulkTables<double>{D.pinvH, D.oct_inv, D.Q,        nullptr,   D.TF,       D.nF,       D.wF,
                                   D.GB,    D.GM,      D.TN,      D.J0,       D.iJ0,      D.Sm,       D.gcl,
                                   D.JF,    D.JE,      D.se_t,     D.se_nang,  D.se_nradL, D.se_nradR,
-                                  m->upload(rfn, err), D.sv_t, m->upload(WFt, err), m->upload(sew, err), m->upload(svw, err),
-                                  m->upload(weta, err), m->upload(iJF, err), m->upload(iJE, err)};
+                                  m->upload(rfn, err), D.sv_t, m->upload(WFt, err), m->upload(sew, err),
+                                  m->upload(svw, err), m->upload(weta, err), m->upload(iJF, err), m->upload(iJE, err)};
   const bool f32 = prec == GEO_FP32_BULK;
   if (f32) {
     geo::BulkTables<float>& b = D.b32;
@@ -792,7 +797,7 @@ int geo_step_adjoint(geo_mesh_t m, double dt, const double* U_in, const double* 
   if (e == cudaSuccess) e = cudaMemcpyAsync(m->adj_fwd.phi, phi_in, F * sizeof(double), cudaMemcpyDeviceToDevice, m->st);
   if (e != cudaSuccess) return cuda_fail(e, "adjoint checkpoint copy");
   // forward intermediates of the checkpoint state; with a team schedule the
-  // predictor is the node team that also stores its Picard iterates, which the
+  // predictor is the ring kernel that also stores its Picard iterates, which the
   // reverse predictor then reads instead of recomputing them
   const bool store = m->dt.predictor != GEO_PRED_ZONE_THREAD;
   for (int s = geo::ST_WENO; s <= geo::ST_ADER && e == cudaSuccess; ++s) {

@@ -7,16 +7,16 @@ namespace geo {
 
 template <int P> struct Dim;
 template <> struct Dim<2> {
-  static constexpr int N = 8, M = 2, NC1 = 3, NC1P = 4, QTRI = 12, NC = 4, NB = 7, NQR = 4, NQS = 4, NQT = 24, NS = 1,
-                       SMAX = 6, NBIN = 3 * NC + NQT + 6, NNZ = 16, NFN = 4, NEN = 2, RL = 2;
+  static constexpr int N = 8, M = 2, NC1 = 3, NC1P = 4, QTRI = 12, NC = 4, NB = 7, NQR = 4, NQS = 4, NQT = 24,
+                       NS = 1, SMAX = 6, NBIN = 3 * NC + NQT + 6, NNZ = 16, NFN = 4, NEN = 2, RL = 2;
 };
 template <> struct Dim<3> {
-  static constexpr int N = 20, M = 3, NC1 = 9, NC1P = 12, QTRI = 60, NC = 10, NB = 16, NQR = 4, NQS = 4, NQT = 24, NS = 2,
-                       SMAX = 26, NBIN = 3 * NC + NQT + 6, NNZ = 96, NFN = 8, NEN = 3, RL = 8;
+  static constexpr int N = 20, M = 3, NC1 = 9, NC1P = 12, QTRI = 60, NC = 10, NB = 16, NQR = 4, NQS = 4, NQT = 24,
+                       NS = 2, SMAX = 26, NBIN = 3 * NC + NQT + 6, NNZ = 96, NFN = 8, NEN = 3, RL = 8;
 };
 template <> struct Dim<4> {
-  static constexpr int N = 32, M = 4, NC1 = 19, NC1P = 20, QTRI = 220, NC = 20, NB = 30, NQR = 9, NQS = 6, NQT = 42, NS = 3,
-                       SMAX = 32, NBIN = 3 * NC + NQT + 6, NNZ = 192, NFN = 12, NEN = 4, RL = 8;
+  static constexpr int N = 32, M = 4, NC1 = 19, NC1P = 20, QTRI = 220, NC = 20, NB = 30, NQR = 9, NQS = 6, NQT = 42,
+                       NS = 3, SMAX = 32, NBIN = 3 * NC + NQT + 6, NNZ = 192, NFN = 12, NEN = 4, RL = 8;
 };
 
 // Reference-element constants of one order in the bulk arithmetic type R, kept

@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(Team<P>::ZB * Dim<P>::N, TeamOcc<P, R>::MINB)
                 double dt) {
   using Dm = Dim<P>;
   constexpr int N = Dm::N, M = Dm::M, NC1 = Dm::NC1, NC = Dm::NC, NQT = Dm::NQT, NS = Dm::NS,
-                NBIN = Dm::NBIN, NR = 3 + 3 * Dm::N, ZB = Team<P>::ZB, NT = ZB * N;
+                NBIN = Dm::NBIN, ZB = Team<P>::ZB, NT = ZB * N;
   __shared__ TeamSmem<P, R> S;
   const RefConst<P, R>& K = RC<P, R>::get();
   const BulkTables<R>& BT = bulk<R>(T);

@@ -57,8 +57,9 @@ def test_cfl_refuses_what_fp32_cannot_tell(part, b):
 # units.  At 4^-272 the product of density and energy is below the range of FP64 (so are
 # the squares of the momentum, which is why the unphysical state stops at 4^-200), at 4^250
 # it is near the upper end
-@pytest.mark.parametrize("k,thermal,flagged", [(-272, 1.0, False), (-200, 1.0, False), (0, 1.0, False), (250, 1.0, False),
-                                               (-200, -1e-6, True), (0, -1e-6, True), (250, -1e-6, True)])
+@pytest.mark.parametrize("k,thermal,flagged", [(-272, 1.0, False), (-200, 1.0, False), (0, 1.0, False),
+                                               (250, 1.0, False), (-200, -1e-6, True), (0, -1e-6, True),
+                                               (250, -1e-6, True)])
 def test_state_flag_in_other_units(k, thermal, flagged):
     from paper_1905_02504_gb300 import geomhd
     from paper_1905_02504_gb300.inputs import make_problem
