@@ -128,8 +128,8 @@ def test_state_flag_near_vacuum(thermal, flagged, prec):
     m.close()
 
 
-# 37,500 faces and 41,256 edges lie on different sides of the size from which one thread
-# takes a whole face or edge: timing the stages must not move a bit of the result
+# timing the stages (a launch each) must not move a bit of the result; 37,500 faces and
+# 41,256 edges lie on the two sides of the size rule, which goes by faces
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("n,nr,p", [(25, 3, 3), (3, 3, 3), (8, 8, 2), (5, 3, 4)])
 def test_stage_timing_leaves_the_result_alone(n, nr, p, prec):
